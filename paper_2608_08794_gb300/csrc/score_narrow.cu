@@ -354,7 +354,7 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       units += ctas;
       units8 += ctas8;
       logit_base += static_cast<int64_t>(sq.rows) * sq.lstride;
-      part_base += static_cast<int64_t>(sq.rows) * ctas8;
+      part_base += static_cast<int64_t>(sq.rows) * sq.nparts;   // the running kernel's partials, not the other's
       lse_base += sq.rows;
       rows_all += sq.rows;
       max_rows = sq.rows > max_rows ? sq.rows : max_rows;

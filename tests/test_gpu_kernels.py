@@ -113,6 +113,18 @@ def test_narrow_path_scores_match_oracle(ap, lens, nqs, hq, hkv):
     assert got.tobytes() == again.tobytes()
 
 
+def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap):
+    """The general logits kernel writes one partial per 256 keys.  A batch of more than 256 keys per
+    SM (38,912 tokens on 152 SMs) is one where a sequence has more of those than the tensor-core
+    kernel's chunks: every sequence's partials need their own place all the same."""
+    lens, nqs, hq, hkv = [21000, 17011, 9003], [2, 3, 1], 28, 4
+    rng = np.random.default_rng(77)
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv)
+    ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv)
+    check_scores(got, ref, strict_rel=2e-3)
+
+
 @pytest.mark.parametrize("lens,nqs,hq,hkv", SHAPES)
 def test_scores_match_oracle(ap, lens, nqs, hq, hkv):
     rng = np.random.default_rng(sum(lens) + hq)
