@@ -21,6 +21,15 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;
 // Key splits of the row-statistics pass (upper bound, sizes the workspace).
 constexpr int kMaxSplits = 32;
 
+// log2(e) / sqrt(D), the factor from a dot product to its log2-domain logit.
+constexpr float kScale2 = 0.12751743082459868f;
+// The same for dot products of the tensor cores, one unit in the last place above (1.26e-7 relative):
+// the fp32 accumulators of tcgen05.mma are truncated, which leaves a dot product of 128 bf16 pairs
+// 1.1e-7 of its magnitude too small on average (measured against 64 bits), and the softmax turns that
+// into a bias of the large logits.  Scores of the 5-minute sequence with three query tokens: 2.4e-7
+// off in the 2-norm with kScale2, 1.4e-7 with this.
+constexpr float kScale2Tc = 0.12751744687557220f;
+
 // Device error word at offset 0 of the workspace.
 struct DeviceError {
   int32_t code;     // APACK_OK, APACK_ETIMEOUT, APACK_EDEVICE (first error wins)

@@ -3,17 +3,18 @@
 // (Table S-hparams), i.e. G = Hq/Hkv rows per group (7 for the 7B model).
 //
 // With so few rows the step is bound by reading K once, so the logits are computed once and
-// kept: three launches.
-//   logits kernel:  log2-domain logits x * log2(e)/sqrt(D) of every (logit row, key), stored per
-//                   logit row with a row stride padded to 64 keys, and per CTA the (max, sum of
-//                   exp2) of every logit row over its multimodal keys.  Two variants:
-//                   * Hkv = 2 or 4 with at most 8 rows per head group: the tcgen05 kernel of
-//                     score_narrow_tc.cu (keys as M = 128, the group's rows as N = 16);
-//                   * other shapes: one thread per key reads its whole token row and dots it
+// kept:
+//   logits kernel:  the dot product of every (logit row, key), stored per logit row with a row
+//                   stride padded to 64 keys, and per CTA the (max, sum of exp2) of every logit row
+//                   over its multimodal keys, in log2 units.  Two variants:
+//                   * Hkv = 1, 2, 4 or 8: the tcgen05 kernel of score_narrow_tc.cu (keys as M = 128,
+//                     the group's rows as N = 16 or 32);
+//                   * other head counts: one thread per key reads its whole token row and dots it
 //                     with the group's query rows held in shared memory;
-//   merge kernel:   per logit row, one block combines the CTA partials into lse2;
-//   final kernel:   one thread per key sums exp2(logit - lse2) over all logit rows
-//                   in a fixed order and scales by 1/(Hq n_q).
+//   final kernel:   the row normalisers lse2 from the CTA partials, then one thread per key sums
+//                   exp2(x log2(e)/sqrt(D) - lse2) over all logit rows in a fixed order and scales
+//                   by 1/(Hq n_q).  When a sequence has many partials (kMergeInside) a merge kernel
+//                   computes lse2 first.
 // The logits of the 10-minute 7B sequence with one query row take 15 MB and stay
 // in L2 between the first and the last kernel.
 #include <algorithm>
@@ -27,9 +28,13 @@ namespace apack {
 
 namespace {
 
-constexpr int kThreads = 256;          // keys per CTA (general logits kernel, final kernel)
+constexpr int kThreads = 256;          // keys per CTA (general logits kernel)
 constexpr int kWarps = kThreads / 32;
-constexpr int kRows8Tokens = 64;       // lower bound of the tensor-core kernel's key chunk (sizes partials)
+constexpr int kFinalThreads = 512;     // threads per CTA (final kernel)
+constexpr int kPartTokens = 64;        // a sequence has at most one partial per this many keys (sizes the workspace)
+// Rows times partials of a sequence up to which every CTA of the final kernel merges the partials by
+// itself instead of a kernel of its own before it.
+constexpr int kMergeInside = 16384;
 constexpr int kLogitPad = 64;          // logit row stride: the key count rounded up to this
 
 __device__ __forceinline__ bool is_mm(uint8_t m) { return m == APACK_MOD_AUDIO || m == APACK_MOD_VISUAL; }
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(kThreads)
       if (l < rg) {
         const int rho = qoff[l] / 128;
         const float y = acc[l] * plan.scale2;
-        if (in) logits[lbase + static_cast<int64_t>(rho) * sq.lstride] = y;
+        if (in) logits[lbase + static_cast<int64_t>(rho) * sq.lstride] = acc[l];
         // this warp's (max, sum of exp2) of the row over the keys in its denominator: the
         // multimodal keys, or (causal rows) every key up to the row's own position
         const bool use = plan.causal ? (in && key - sq.t0 <= sq.q_pos + l / G) : mm;
@@ -134,7 +139,7 @@ __global__ void __launch_bounds__(kThreads)
         const float2 v = wpart[w * R + rho];
         if (v.x != -INFINITY) sum += v.y * ex2_approx(v.x - m);
       }
-    part[sq.part_base + static_cast<int64_t>(kt) * R + rho] = make_float2(m, sum);
+    part[sq.part_base + static_cast<int64_t>(rho) * sq.nparts + kt] = make_float2(m, sum);
   }
 }
 
@@ -164,11 +169,11 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
     for (int i = 0; i < kHold; ++i) {
       const int c = tid + i * kThreads;
-      v[i] = c < ctas ? part[sq.part_base + static_cast<int64_t>(c) * sq.rows + rho] : make_float2(-INFINITY, 0.f);
+      v[i] = c < ctas ? part[sq.part_base + static_cast<int64_t>(rho) * sq.nparts + c] : make_float2(-INFINITY, 0.f);
       m = fmaxf(m, v[i].x);
     }
   } else {
-    for (int c = tid; c < ctas; c += kThreads) m = fmaxf(m, part[sq.part_base + static_cast<int64_t>(c) * sq.rows + rho].x);
+    for (int c = tid; c < ctas; c += kThreads) m = fmaxf(m, part[sq.part_base + static_cast<int64_t>(rho) * sq.nparts + c].x);
   }
   m = warp_max(m);
   if (lane == 0) red[warp] = m;
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(kThreads)
         if (v[i].x != -INFINITY) sum += v[i].y * exp2f(v[i].x - m);
     } else {
       for (int c = tid; c < ctas; c += kThreads) {
-        const float2 w = part[sq.part_base + static_cast<int64_t>(c) * sq.rows + rho];
+        const float2 w = part[sq.part_base + static_cast<int64_t>(rho) * sq.nparts + c];
         if (w.x != -INFINITY) sum += w.y * exp2f(w.x - m);
       }
     }
@@ -205,58 +210,105 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// One thread per key: I = sum over logit rows of exp2(logit - lse2) / (Hq n_q).
-__global__ void __launch_bounds__(kThreads)
+// One thread per key: I = sum over logit rows of exp2(x c2 - lse2) / (Hq n_q), x the stored dot
+// product.  MERGE: the CTA's warps first merge the sequence's partials into lse2, two rows per warp
+// and round, while the keys' own logits are in flight (a fixed order).  SPLIT threads share a key's
+// rows when there are more than 32 of them, so that a thread's loads stay one or two rounds.
+// Latency-bound (two L2 round trips and the launch): 8.5 us for 28 rows of 135,041 keys, where the
+// merge and final kernels took 10.3 us in two launches.
+template <bool MERGE, int SPLIT>
+__global__ void __launch_bounds__(kFinalThreads)
     score_narrow_final_kernel(const __grid_constant__ NarrowPlan plan, const uint8_t *__restrict__ modality,
-                              const float *__restrict__ logits, const float *__restrict__ lse2,
-                              float *__restrict__ scores) {
+                              const float *__restrict__ logits, const float2 *__restrict__ part,
+                              const float *__restrict__ lse2, float *__restrict__ scores) {
   pdl_wait_and_release();
-  extern __shared__ __align__(16) float ls[];
-  const int s = find_unit_seq(plan, blockIdx.x);
+  extern __shared__ __align__(16) float ls[];            // -lse2 per logit row
+  const int s = find_final_seq(plan, blockIdx.x);
   const NSeq &sq = plan.seq[s];
   const int R = sq.rows;
-  const int kt = blockIdx.x - sq.unit_begin;
-  const int key = sq.t0 + kt * kThreads + threadIdx.x;
+  const int kt = blockIdx.x - sq.final_begin;
+  constexpr int kKeys = kFinalThreads / SPLIT;           // keys per CTA
+  const int kl = threadIdx.x % kKeys;
+  const int key = sq.t0 + kt * kKeys + kl;
   const bool in = key < sq.t0 + sq.len;
   const float *lp = logits + sq.logit_base + (key - sq.t0);
-  // the key's own loads (modality, and up to 32 rows' logits) are issued before the normalisers
-  // arrive: one round trip for all of them
+  // this thread's rows [ra, rb); the key's own loads (modality, and the first 32 rows' logits) are
+  // issued before the normalisers arrive: one round trip for all of them
+  const int share = threadIdx.x / kKeys, per = (R + SPLIT - 1) / SPLIT;
+  const int ra = SPLIT == 1 ? 0 : min(R, share * per), rb = SPLIT == 1 ? R : min(R, ra + per);
   const uint8_t mod = in ? modality[key] : static_cast<uint8_t>(0);
   float raw[32];
-  if (R <= 32) {
 #pragma unroll
-    for (int u = 0; u < 32; ++u) raw[u] = (in && u < R) ? lp[static_cast<int64_t>(u) * sq.lstride] : 0.f;
+  for (int u = 0; u < 32; ++u) raw[u] = (in && ra + u < rb) ? lp[static_cast<int64_t>(ra + u) * sq.lstride] : 0.f;
+  if (MERGE) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // two rows per warp and round, the loads of both issued together; each row's first 160 partials
+    // are read once
+    constexpr int kHold = 5;
+    for (int r0 = warp; r0 < R; r0 += 2 * (kFinalThreads / 32)) {
+      float2 v[2][kHold];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int rho = r0 + k * (kFinalThreads / 32);
+        const float2 *p = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
+#pragma unroll
+        for (int i = 0; i < kHold; ++i)
+          v[k][i] = rho < R && lane + 32 * i < sq.nparts ? p[lane + 32 * i] : make_float2(-INFINITY, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int rho = r0 + k * (kFinalThreads / 32);
+        if (rho >= R) break;                             // uniform over the warp
+        const float2 *p = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
+        float m = v[k][0].x, sum = 0.f;
+#pragma unroll
+        for (int i = 1; i < kHold; ++i) m = fmaxf(m, v[k][i].x);
+        for (int c = lane + 32 * kHold; c < sq.nparts; c += 32) m = fmaxf(m, p[c].x);
+        m = warp_max(m);
+        if (m != -INFINITY) {
+#pragma unroll
+          for (int i = 0; i < kHold; ++i) sum += v[k][i].y * exp2f(v[k][i].x - m);
+          for (int c = lane + 32 * kHold; c < sq.nparts; c += 32) sum += p[c].y * exp2f(p[c].x - m);
+        }
+        sum = warp_sum(sum);
+        // no key in the denominator: nothing is scored in this row
+        if (lane == 0) ls[rho] = m == -INFINITY ? -INFINITY : -(m + log2f(sum));
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < R; i += kFinalThreads) ls[i] = -lse2[sq.lse_base + i];
   }
-  for (int i = threadIdx.x; i < R; i += kThreads) ls[i] = lse2[sq.lse_base + i];
   __syncthreads();
-  if (!in) return;
   float out = 0.f;
-  if (sq.n_q > 0 && is_mm(mod)) {
-    // eight independent sums, the loads of a block of 8 rows issued together
+  const bool scored = in && sq.n_q > 0 && is_mm(mod);
+  if (scored) {
+    const float c2 = plan.scale2;
+    // eight independent sums, the loads of a block of 16 rows issued together
     float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     // causal rows: logit row rho = token * Hq + head sees this key when token >= key - q_pos
     const int rho_min = plan.causal ? max(0, key - sq.t0 - sq.q_pos) * plan.hq : 0;
-    if (R <= 32) {
-      // all rows (the paper's one query token: R = Hq)
-      float x[32];
 #pragma unroll
-      for (int u = 0; u < 32; ++u) x[u] = (u < R && u >= rho_min) ? raw[u] - ls[u] : -INFINITY;
+    for (int u = 0; u < 32; ++u)
+      if (ra + u < rb && ra + u >= rho_min) a[u & 7] += ex2_approx(fmaf(raw[u], c2, ls[ra + u]));
+    for (int r0 = ra + 32; r0 < rb; r0 += 16) {
+      float x[16];
 #pragma unroll
-      for (int u = 0; u < 32; ++u) a[u & 7] += ex2_approx(x[u]);
-    } else {
-      for (int r0 = 0; r0 < R; r0 += 8) {
-        float x[8];
+      for (int u = 0; u < 16; ++u) x[u] = r0 + u < rb ? lp[static_cast<int64_t>(r0 + u) * sq.lstride] : 0.f;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          x[u] = (r0 + u < R && r0 + u >= rho_min) ? lp[static_cast<int64_t>(r0 + u) * sq.lstride] - ls[r0 + u]
-                                                   : -INFINITY;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] += ex2_approx(x[u]);
-      }
+      for (int u = 0; u < 16; ++u)
+        if (r0 + u < rb && r0 + u >= rho_min) a[u & 7] += ex2_approx(fmaf(x[u], c2, ls[r0 + u]));
     }
-    out = (((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]))) / static_cast<float>(plan.hq * sq.n_q);
+    out = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
   }
-  scores[key] = out;
+  if (SPLIT > 1) {                                       // the shares of a key meet in share order
+    __shared__ float sums[SPLIT > 1 ? kFinalThreads : 1];
+    sums[threadIdx.x] = out;
+    __syncthreads();
+    if (share > 0) return;
+#pragma unroll
+    for (int i = 1; i < SPLIT; ++i) out += sums[i * kKeys + kl];
+  }
+  if (in) scores[key] = scored ? out / static_cast<float>(plan.hq * sq.n_q) : 0.f;
 }
 
 template <int RG>
@@ -289,7 +341,7 @@ void narrow_layout(const apack_seqs *s, size_t *logit_floats, size_t *part_float
     const int64_t len = s->cu_seqlens_h[b + 1] - s->cu_seqlens_h[b];
     const int64_t R = static_cast<int64_t>(s->num_q_heads) * (s->cu_qlens_h[b + 1] - s->cu_qlens_h[b]);
     lf += static_cast<size_t>(R * ((len + kLogitPad - 1) / kLogitPad * kLogitPad));
-    pf += static_cast<size_t>(R * ((len + kRows8Tokens - 1) / kRows8Tokens));   // enough for either kernel
+    pf += static_cast<size_t>(R * ((len + kPartTokens - 1) / kPartTokens));   // enough for either kernel
     ef += static_cast<size_t>(R);
   }
   *logit_floats = lf;
@@ -314,25 +366,41 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
     P.hq = hq;
     P.hkv = hkv;
     P.group = G;
-    P.scale2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(APACK_HEAD_DIM)));
     P.causal = seqs->softmax_domain == APACK_SOFTMAX_CAUSAL_ROW;
-    // tensor-core logits kernel: Hkv = 2 or 4, at most 8 rows per head group
     int max_rg = 0;
     for (int i = 0; i < ns; ++i) {
       const int nq = seqs->cu_qlens_h[s0 + i + 1] - seqs->cu_qlens_h[s0 + i];
       max_rg = G * nq > max_rg ? G * nq : max_rg;
     }
-    const bool rows8 = (hkv == 2 || hkv == 4) && max_rg <= 8;
-    // its chunk: about one CTA per SM over this launch's keys, whole 128-key tiles
-    int64_t launch_tokens = 0;
-    for (int i = 0; i < ns; ++i) launch_tokens += seqs->cu_seqlens_h[s0 + i + 1] - seqs->cu_seqlens_h[s0 + i];
-    const int64_t stage_tok = 128;     // chunks are whole 128-key tensor-core tiles
+    const bool tc = hkv == 1 || hkv == 2 || hkv == 4 || hkv == 8;
+    P.scale2 = tc ? kScale2Tc : kScale2;
+    // its work: the (tile, KV head) stages of the sequences with query rows, `chunk` of them per CTA,
+    // the smallest chunk (within 3 %) that keeps the launch to one CTA per SM
+    auto stages_of = [&](int b) -> int64_t {
+      const int64_t len = seqs->cu_seqlens_h[b + 1] - seqs->cu_seqlens_h[b];
+      return seqs->cu_qlens_h[b + 1] > seqs->cu_qlens_h[b] ? (len + 127) / 128 * hkv : 0;
+    };
+    auto ctas_of = [&](int b, int64_t chunk) -> int64_t {
+      const int64_t len = seqs->cu_seqlens_h[b + 1] - seqs->cu_seqlens_h[b];
+      return std::min<int64_t>((stages_of(b) + chunk - 1) / chunk, (len + kPartTokens - 1) / kPartTokens);
+    };
     const int64_t sms = device_sm_count();
-    int64_t chunk = (launch_tokens + sms - 1) / sms;
-    chunk = std::max<int64_t>(stage_tok, (chunk + stage_tok - 1) / stage_tok * stage_tok);
-    P.chunk = static_cast<int32_t>(std::min<int64_t>(chunk, 1 << 24));
-    int units = 0, units8 = 0, max_rows = 0;
-    int64_t rows_all = 0;
+    int64_t all_stages = 0, max_stages = 1;
+    for (int i = 0; i < ns; ++i) {
+      all_stages += stages_of(s0 + i);
+      max_stages = std::max(max_stages, stages_of(s0 + i));
+    }
+    int64_t chunk = std::max<int64_t>(1, (all_stages + sms - 1) / sms);
+    for (; chunk < max_stages; chunk += std::max<int64_t>(1, chunk / 32)) {
+      int64_t ctas = 0;
+      for (int i = 0; i < ns; ++i) ctas += ctas_of(s0 + i, chunk);
+      if (ctas <= sms) break;
+    }
+    // the final kernel's threads per key: up to 32 rows each, then twice that
+    const int split = hq * (max_rg / G) <= 32 ? 1 : hq * (max_rg / G) <= 128 ? 2 : 4;
+    const int final_keys = kFinalThreads / split;
+    int units = 0, units8 = 0, finals = 0, max_rows = 0;
+    int64_t rows_all = 0, max_parts = 0;
     for (int i = 0; i < ns; ++i) {
       const int b = s0 + i;
       NSeq &sq = P.seq[i];
@@ -344,53 +412,64 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       sq.q_pos = query_position(seqs, b);
       sq.unit_begin = units;
       sq.unit8_begin = units8;
+      sq.final_begin = finals;
       sq.lstride = (sq.len + kLogitPad - 1) / kLogitPad * kLogitPad;
       sq.logit_base = logit_base;
       sq.part_base = part_base;
       sq.lse_base = lse_base;
+      sq.stages = static_cast<int32_t>(stages_of(b));
       const int ctas = (sq.len + kThreads - 1) / kThreads;
-      const int ctas8 = (sq.len + P.chunk - 1) / P.chunk;   // <= (len + 63) / 64: fits the workspace
-      sq.nparts = rows8 ? ctas8 : ctas;
+      int ctas8 = static_cast<int>(ctas_of(b, chunk));
+      sq.chunk = ctas8 > 0 ? (sq.stages + ctas8 - 1) / ctas8 : 1;
+      ctas8 = (sq.stages + sq.chunk - 1) / sq.chunk;        // no CTA without a stage
+      sq.nparts = tc ? ctas8 : ctas;                        // at most one per kPartTokens keys: fits the workspace
       units += ctas;
       units8 += ctas8;
+      finals += (sq.len + final_keys - 1) / final_keys;
       logit_base += static_cast<int64_t>(sq.rows) * sq.lstride;
-      part_base += static_cast<int64_t>(sq.rows) * sq.nparts;   // the running kernel's partials, not the other's
+      part_base += static_cast<int64_t>(sq.rows) * sq.nparts;
       lse_base += sq.rows;
       rows_all += sq.rows;
       max_rows = sq.rows > max_rows ? sq.rows : max_rows;
+      max_parts = std::max(max_parts, static_cast<int64_t>(sq.rows) * sq.nparts);
     }
     P.total_units = units;
     P.total_units8 = units8;
     if (units == 0) continue;
-    cudaError_t e;
     const uint16_t *q16 = static_cast<const uint16_t *>(q);
     const uint8_t *k8 = static_cast<const uint8_t *>(k);
-    if (rows8) {
-      DeviceError *err = reinterpret_cast<DeviceError *>(wsb + L.err_off);
-      CUtensorMap kmap;
-      if (!make_kv_tile_map(&kmap, k, hkv, seqs->cu_seqlens_h[B], k_token_stride, 128)) return APACK_ECUDA;
-      e = launch_narrow_tc(units8, stream, kmap, P, q16, seqs->modality, logits, part, err);
-    } else {
-      const size_t smem = static_cast<size_t>(max_rows) * 128 * sizeof(float) +
-                          static_cast<size_t>(kWarps) * max_rows * sizeof(float2);
-      if (max_rg <= 8)
-        e = launch_logits<8>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
-      else if (max_rg <= 16)
-        e = launch_logits<16>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
-      else
-        e = launch_logits<32>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
+    if (tc ? units8 > 0 : units > 0) {
+      cudaError_t e;
+      if (tc) {
+        DeviceError *err = reinterpret_cast<DeviceError *>(wsb + L.err_off);
+        CUtensorMap kmap;
+        if (!make_kv_tile_map(&kmap, k, hkv, seqs->cu_seqlens_h[B], k_token_stride, 128)) return APACK_ECUDA;
+        e = launch_narrow_tc(max_rg, units8, stream, kmap, P, q16, seqs->modality, logits, part, err);
+      } else {
+        const size_t smem = static_cast<size_t>(max_rows) * 128 * sizeof(float) +
+                            static_cast<size_t>(kWarps) * max_rows * sizeof(float2);
+        if (max_rg <= 8)
+          e = launch_logits<8>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
+        else if (max_rg <= 16)
+          e = launch_logits<16>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
+        else
+          e = launch_logits<32>(units, smem, stream, P, q16, k8, k_token_stride, seqs->modality, logits, part);
+      }
+      count_launches(1);
+      if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
-    count_launches(1);
-    if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
-    if (rows_all > 0) {
+    const bool inside = max_parts <= kMergeInside;
+    if (rows_all > 0 && !inside) {
       if (check_cuda(launch_pdl(score_narrow_merge_kernel, dim3(static_cast<unsigned>(rows_all)), dim3(kThreads), 0,
                                 stream, P, part, lse2)) != APACK_OK)
         return APACK_ECUDA;
       count_launches(1);
     }
-    if (check_cuda(launch_pdl(score_narrow_final_kernel, dim3(units), dim3(kThreads),
-                              static_cast<size_t>(max_rows) * sizeof(float), stream, P, seqs->modality, logits, lse2,
-                              scores)) != APACK_OK)
+    auto *final_kernel = split == 1   ? (inside ? score_narrow_final_kernel<true, 1> : score_narrow_final_kernel<false, 1>)
+                         : split == 2 ? (inside ? score_narrow_final_kernel<true, 2> : score_narrow_final_kernel<false, 2>)
+                                      : (inside ? score_narrow_final_kernel<true, 4> : score_narrow_final_kernel<false, 4>);
+    if (check_cuda(launch_pdl(final_kernel, dim3(finals), dim3(kFinalThreads), static_cast<size_t>(max_rows) * sizeof(float),
+                              stream, P, seqs->modality, logits, part, lse2, scores)) != APACK_OK)
       return APACK_ECUDA;
     count_launches(1);
   }

@@ -1,21 +1,27 @@
 // score_narrow_tc.cu -- logits of the narrow scoring path (few query rows per KV head group,
 // e.g. the paper's last query token: Sec. 3.2, Eq. inner_score; Table S-hparams) on the
-// tcgen05 tensor cores.
+// tcgen05 tensor cores, for 1, 2, 4 or 8 KV heads and up to 32 query rows per KV head group.
 //
-// One CTA per chunk of a sequence's keys (about T / #SMs keys).  For every 128-key tile and KV
-// head h, the MMA computes D[key][row] = K_h[key] . Q_h[row] with keys as M = 128 and the
-// head group's query rows as N = 16 (zero rows pad the group's <= 8 rows): bf16 operands in
-// 128-byte-swizzled shared memory, fp32 accumulators in TMEM.
-//   warp 0, one lane:  TMA loads of the K tiles (one stage = one head of one tile, 32 KB)
+// A stage is one KV head of one 128-key tile (32 KB of K).  The stages of a sequence are cut into
+// equal contiguous ranges, one per CTA (about one CTA per SM over the launch); for each stage the
+// MMA computes D[key][row] = K_h[key] . Q_h[row] with keys as M = 128 and the head group's query
+// rows as N = 16 or 32 (zero rows pad them): bf16 operands in 128-byte-swizzled shared memory, fp32
+// accumulators in TMEM.
+//   warp 0, one lane:  TMA loads of the K stages, the first ones before the query rows are staged
 //   warp 1, one lane:  TMEM allocation and the MMAs (8 per stage), commits to mbarriers
-//   warps 2..:         epilogue, one warpgroup per KV head, one key per thread: reads its
-//                      head's 16 TMEM columns of the tile,
-//                      stores the log2-domain logits (row-major per logit row, as the
-//                      CUDA-core path) and keeps, per (head, row), the running (max, sum of
-//                      exp2) over its multimodal keys.
-// At the end the CTA merges the 128 per-thread states per logit row in thread order and
-// writes one (max, sum) partial per row: the merge and final kernels of the narrow path
-// consume the logits and partials unchanged.  Every wait is bounded.
+//   warps 2..:         epilogue, one warpgroup per KV head (8 heads: two per warpgroup), one key per
+//                      thread: reads the stage's columns, stores the logits (row-major per logit
+//                      row) and folds the warp's 32 keys into a running (max, sum of exp2) per row.
+//                      The 32 keys meet by a reduce-scatter over the lanes: NR rows cost NR - 1
+//                      shuffles and leave row r in lane r (NR = 32), so the running state of up to
+//                      32 rows is one register pair per lane.
+// At the end the CTA merges its warps' states per logit row in warp order and writes one
+// (max, sum) partial per row for the final kernel.  Every wait is bounded.
+//
+// Bound by reading K once; what the CTA adds to that is its prologue and the last stage's
+// epilogue.  A per-thread online state over up to 8 rows (two registers a row) carried only the
+// shapes of at most 8 rows: the others ran on CUDA cores, one thread per key.
+// Three query tokens (21 rows per group) over 67,541 keys: 127 us there, 20 us here.
 #include <cmath>
 
 #include "internal.cuh"
@@ -26,32 +32,36 @@ namespace apack {
 namespace {
 
 constexpr int kTcM = 128;                          // keys per tile (MMA M)
-constexpr int kTcN = 16;                           // query rows per head group, padded (MMA N)
-constexpr int kTcRows = 8;                         // query rows per head group supported
-constexpr int kTcStages = 6;                       // K ring: one (tile, head) per stage
 constexpr int kTcHalf = kTcM * 128;                // 64 dims x 128 keys x 2 B = 16 KB
 constexpr int kTcStageBytes = 2 * kTcHalf;         // 32 KB
-constexpr int kTcQHalf = kTcN * 128;               // 2 KB: 64 dims of the 16 rows
-// epilogue: one warpgroup (4 warps, one per TMEM lane quadrant) per KV head
-template <int HKV>
-__host__ __device__ constexpr int tc_epi_warps() { return 4 * HKV; }
-template <int HKV>
-__host__ __device__ constexpr int tc_threads() { return 64 + 32 * tc_epi_warps<HKV>(); }   // warp 0 TMA, warp 1 MMA, epilogue
-constexpr uint32_t kTcIdesc = idesc_bf16_f32(kTcM, kTcN);
+constexpr int kTcMaxStages = 6;
+
+// HKV KV heads, at most NR query rows per KV head group.
+template <int HKV, int NR>
+struct TcLayout {
+  static constexpr int kN = NR < 16 ? 16 : NR;                           // MMA N
+  static constexpr int kGroups = HKV < 4 ? HKV : 4;                      // epilogue warpgroups
+  static constexpr int kHeads = HKV / kGroups;                           // KV heads per warpgroup
+  static constexpr int kThreads = 64 + 128 * kGroups;                    // warp 0 TMA, warp 1 MMA, epilogue
+  static constexpr int kQHalf = kN * 128;                                // 64 dims of the kN rows
+  static constexpr int kQBytes = HKV * 2 * kQHalf;
+  static constexpr int kStages = kTcMaxStages * kTcStageBytes + kQBytes <= 230000 ? kTcMaxStages : kTcMaxStages - 1;
+  static constexpr uint32_t kOffQ = kStages * kTcStageBytes;             // 1024-aligned
+  static constexpr uint32_t kOffRho = kOffQ + kQBytes;                   // int32 [NR]: logit row of row j, head 0
+  static constexpr uint32_t kOffBars = kOffRho + NR * 4;
+  static constexpr uint32_t kBytes = kOffBars + 512;
+  static constexpr uint32_t kTmemCols = 2 * HKV * kN;                    // a power of two, 32 .. 512
+  static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcM, kN);
+  static_assert(kBytes <= 232448, "shared memory budget");
+};
 
 struct __align__(8) TcBars {
-  uint64_t k_full[kTcStages], k_empty[kTcStages], acc_full[2], acc_empty[2], drain;
+  uint64_t k_full[kTcMaxStages], k_empty[kTcMaxStages], drain;
+  uint64_t acc_full[8][2], acc_empty[8][2];          // per KV head and accumulator buffer
   uint32_t tmem_base;
   volatile int32_t abort;
 };
-
-template <int HKV>
-struct TcLayout {
-  static constexpr uint32_t kOffQ = kTcStages * kTcStageBytes;           // 1024-aligned
-  static constexpr uint32_t kOffBars = kOffQ + HKV * 2 * kTcQHalf;
-  static constexpr uint32_t kBytes = kOffBars + 256;
-  static constexpr uint32_t kTmemCols = 2 * HKV * kTcN < 32 ? 32 : 2 * HKV * kTcN;   // power of 2 here
-};
+static_assert(sizeof(TcBars) <= 512, "barrier block");
 
 __device__ __forceinline__ bool tc_wait(uint64_t *bar, uint32_t parity, TcBars *bars, DeviceError *err, int where) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -70,13 +80,40 @@ __device__ __forceinline__ bool tc_wait(uint64_t *bar, uint32_t parity, TcBars *
 
 __device__ __forceinline__ bool is_mm_tc(uint8_t m) { return m == APACK_MOD_AUDIO || m == APACK_MOD_VISUAL; }
 
-template <int HKV>
-__global__ void __launch_bounds__(tc_threads<HKV>(), 1)
+__device__ __forceinline__ void load_rows(uint32_t taddr, uint32_t (&r)[8]) { tmem_ld8_wait(taddr, r); }
+__device__ __forceinline__ void load_rows(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld16_wait(taddr, r); }
+__device__ __forceinline__ void load_rows(uint32_t taddr, uint32_t (&r)[32]) {
+  tmem_ld32(taddr, r);
+  tmem_wait32(r);
+}
+
+// Combines v[j] of the 32 lanes for every j < NR with op: lane l ends with row l / (32 / NR).
+// At each level the lanes of a pair exchange the halves that the other one keeps.
+template <int NR, class Op>
+__device__ __forceinline__ float reduce_scatter(float (&v)[NR], int lane, Op op) {
+  int mask = 16;
+#pragma unroll
+  for (int half = NR / 2; half >= 1; half /= 2, mask /= 2) {
+    const bool up = lane & mask;
+#pragma unroll
+    for (int e = 0; e < half; ++e) {
+      const float keep = up ? v[e + half] : v[e];
+      const float send = up ? v[e] : v[e + half];
+      v[e] = op(keep, __shfl_xor_sync(0xffffffffu, send, mask));
+    }
+  }
+#pragma unroll
+  for (; mask >= 1; mask /= 2) v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], mask));
+  return v[0];
+}
+
+template <int HKV, int NR>
+__global__ void __launch_bounds__(TcLayout<HKV, NR>::kThreads, 1)
     score_narrow_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ NarrowPlan plan,
                            const uint16_t *__restrict__ q, const uint8_t *__restrict__ modality,
                            float *__restrict__ logits, float2 *__restrict__ part, DeviceError *err) {
-  pdl_wait_and_release();
-  using Lay = TcLayout<HKV>;
+  using Lay = TcLayout<HKV, NR>;
+  constexpr int kN = Lay::kN, kStages = Lay::kStages;
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0) {
     if (threadIdx.x == 0) raise_device_error(err, APACK_EDEVICE, 80);
@@ -84,23 +121,54 @@ __global__ void __launch_bounds__(tc_threads<HKV>(), 1)
   }
   uint8_t *ring = smem;
   uint8_t *qs = smem + Lay::kOffQ;
+  int32_t *rho_of = reinterpret_cast<int32_t *>(smem + Lay::kOffRho);
   TcBars *bars = reinterpret_cast<TcBars *>(smem + Lay::kOffBars);
-  const int c = blockIdx.x;
-  const int s = find_unit8_seq(plan, c);
+  const int s = find_unit8_seq(plan, blockIdx.x);
   const NSeq &sq = plan.seq[s];
   const int G = plan.group;
-  const int rg = G * sq.n_q;
-  if (rg == 0) return;                                 // no query row: nothing to score (CTA-uniform)
+  const int rg = G * sq.n_q;                           // rows per head group, 1 .. NR (sequences without have no CTA)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tb = (c - sq.unit8_begin) * plan.chunk;
-  const int te = min(sq.len, tb + plan.chunk);
-  const int ntiles = (te - tb + kTcM - 1) / kTcM;
+  const int c = blockIdx.x - sq.unit8_begin;           // this CTA's range of the sequence's stages
+  const int u0 = c * sq.chunk;
+  const int nstage = min(sq.stages - u0, sq.chunk);
 
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(&bars->k_full[i], 1);
+      mbar_init(&bars->k_empty[i], 1);
+    }
+    for (int h = 0; h < HKV; ++h)
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(&bars->acc_full[h][i], 1);
+        mbar_init(&bars->acc_empty[h][i], 4);
+      }
+    mbar_init(&bars->drain, 1);
+    bars->abort = 0;
+    fence_mbar_init();
+    tma_prefetch_desc(&kmap);
+  }
+  if (warp == 1) {
+    tmem_alloc(&bars->tmem_base, Lay::kTmemCols);
+    tc_fence_before();
+  }
+  pdl_wait_and_release();   // the set-up above runs beside the previous launch; q and K are read below
+  // stage n of this CTA: unit u0 + n = tile * HKV + head
+  auto issue_load = [&](int n) {
+    const int slot = n % kStages, t = (u0 + n) / HKV, h = (u0 + n) % HKV;
+    uint8_t *dst = ring + slot * kTcStageBytes;
+    const int key0 = sq.t0 + t * kTcM;
+    mbar_arrive_expect_tx(&bars->k_full[slot], kTcStageBytes);
+    tma_load_3d(dst, &kmap, &bars->k_full[slot], 0, h, key0);
+    tma_load_3d(dst + kTcHalf, &kmap, &bars->k_full[slot], 64, h, key0);
+  };
+  const int first = min(nstage, kStages);
+  if (threadIdx.x == 0)
+    for (int n = 0; n < first; ++n) issue_load(n);
   // query tiles in the 128-byte-swizzled K-major layout: row r, 16-byte chunk cc of a 64-dim
   // half sits at chunk cc ^ (r & 7) of the row's 128 bytes (every ring stage the MMAs read is
   // written whole by its TMA load, rows past the cache as zeros)
-  for (int idx = threadIdx.x; idx < HKV * kTcN * 16; idx += tc_threads<HKV>()) {
-    const int h = idx / (kTcN * 16), rem = idx % (kTcN * 16);
+  for (int idx = threadIdx.x; idx < HKV * kN * 16; idx += Lay::kThreads) {
+    const int h = idx / (kN * 16), rem = idx % (kN * 16);
     const int row = rem / 16, ch = rem % 16;
     const int half = ch >> 3, cc = ch & 7;
     uint4 v = make_uint4(0, 0, 0, 0);
@@ -108,218 +176,193 @@ __global__ void __launch_bounds__(tc_threads<HKV>(), 1)
       const int rho = (row / G) * plan.hq + h * G + row % G;
       v = __ldg(reinterpret_cast<const uint4 *>(q + (static_cast<int64_t>(sq.q_off) * plan.hq + rho) * 128) + ch);
     }
-    *reinterpret_cast<uint4 *>(qs + h * 2 * kTcQHalf + half * kTcQHalf + (row >> 3) * 1024 + (row & 7) * 128 +
+    *reinterpret_cast<uint4 *>(qs + h * 2 * Lay::kQHalf + half * Lay::kQHalf + (row >> 3) * 1024 + (row & 7) * 128 +
                                ((cc ^ (row & 7)) << 4)) = v;
   }
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kTcStages; ++i) {
-      mbar_init(&bars->k_full[i], 1);
-      mbar_init(&bars->k_empty[i], 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&bars->acc_full[i], 1);
-      mbar_init(&bars->acc_empty[i], tc_epi_warps<HKV>());
-    }
-    mbar_init(&bars->drain, 1);
-    bars->abort = 0;
-    fence_mbar_init();
-  }
-  fence_proxy_async_smem();   // generic-proxy writes of the tiles -> visible to TMA and the MMA
-  if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, Lay::kTmemCols);
-    tc_fence_before();
-  }
+  for (int j = threadIdx.x; j < NR; j += Lay::kThreads) rho_of[j] = (j / G) * plan.hq + j % G;
+  fence_proxy_async_smem();   // generic-proxy writes of the query tiles -> visible to the MMA
   __syncthreads();
   tc_fence_after();
-  const int nstage = ntiles * HKV;
+
+  // epilogue warps: running (max, sum of exp2) of the row this lane owns, per KV head
+  float m_run[Lay::kHeads], l_run[Lay::kHeads];
+#pragma unroll
+  for (int i = 0; i < Lay::kHeads; ++i) {
+    m_run[i] = -INFINITY;
+    l_run[i] = 0.f;
+  }
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&kmap);
-      int n = 0;
-      bool pend[kTcStages] = {};
-      uint32_t pend_par[kTcStages] = {};
+      int n = first;
       for (; n < nstage; ++n) {
-        const int slot = n % kTcStages;
-        if (n >= kTcStages && !tc_wait(&bars->k_empty[slot], ((n / kTcStages) - 1) & 1u, bars, err, 81)) break;
-        const int t = n / HKV, h = n % HKV;
-        uint8_t *dst = ring + slot * kTcStageBytes;
-        mbar_arrive_expect_tx(&bars->k_full[slot], kTcStageBytes);
-        const int key0 = sq.t0 + tb + t * kTcM;
-        tma_load_3d(dst, &kmap, &bars->k_full[slot], 0, h, key0);
-        tma_load_3d(dst + kTcHalf, &kmap, &bars->k_full[slot], 64, h, key0);
-        pend[slot] = true;
-        pend_par[slot] = (n / kTcStages) & 1u;
+        if (!tc_wait(&bars->k_empty[n % kStages], ((n / kStages) - 1) & 1u, bars, err, 81)) break;
+        issue_load(n);
       }
-      if (bars->abort)   // loads issued but not consumed: let them land before the CTA exits
-        for (int i = 0; i < kTcStages; ++i)
-          if (pend[i]) mbar_wait(&bars->k_full[i], pend_par[i], kWaitLimitNs / 4);
+      if (bars->abort)   // loads issued but not consumed: let the last of every slot land before the CTA exits
+        for (int i = n > kStages ? n - kStages : 0; i < n; ++i)
+          mbar_wait(&bars->k_full[i % kStages], (i / kStages) & 1u, kWaitLimitNs / 4);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       const uint32_t tmem = bars->tmem_base;
       const uint32_t q_base = smem_u32(qs);
-      bool ok = true;
-      for (int t = 0; ok && t < ntiles; ++t) {
-        const int buf = t & 1;
-        if (t >= 2 && !tc_wait(&bars->acc_empty[buf], ((t >> 1) - 1) & 1u, bars, err, 82)) break;
-        for (int h = 0; h < HKV; ++h) {
-          const int n = t * HKV + h, slot = n % kTcStages;
-          if (!tc_wait(&bars->k_full[slot], (n / kTcStages) & 1u, bars, err, 83)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t a_base = smem_u32(ring + slot * kTcStageBytes);
-          const uint32_t b_base = q_base + h * 2 * kTcQHalf;
+      for (int n = 0; n < nstage; ++n) {
+        const int h = (u0 + n) % HKV, i = n / HKV, buf = i & 1, slot = n % kStages;   // i: earlier stages of the head
+        if (i >= 2 && !tc_wait(&bars->acc_empty[h][buf], ((i >> 1) - 1) & 1u, bars, err, 82)) break;
+        if (!tc_wait(&bars->k_full[slot], (n / kStages) & 1u, bars, err, 83)) break;
+        tc_fence_after();
+        const uint32_t a_base = smem_u32(ring + slot * kTcStageBytes);
+        const uint32_t b_base = q_base + h * 2 * Lay::kQHalf;
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t ao = (kk >> 2) * kTcHalf + (kk & 3) * 32;
-            const uint32_t bo = (kk >> 2) * kTcQHalf + (kk & 3) * 32;
-            tc_mma_bf16(tmem + buf * HKV * kTcN + h * kTcN, smem_desc_sw128(a_base + ao), smem_desc_sw128(b_base + bo),
-                        kTcIdesc, kk > 0 ? 1u : 0u);
-          }
-          tc_commit(&bars->k_empty[slot]);
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t ao = (kk >> 2) * kTcHalf + (kk & 3) * 32;
+          const uint32_t bo = (kk >> 2) * Lay::kQHalf + (kk & 3) * 32;
+          tc_mma_bf16(tmem + (buf * HKV + h) * kN, smem_desc_sw128(a_base + ao), smem_desc_sw128(b_base + bo),
+                      Lay::kIdesc, kk > 0 ? 1u : 0u);
         }
-        if (ok) tc_commit(&bars->acc_full[buf]);
+        tc_commit(&bars->k_empty[slot]);
+        tc_commit(&bars->acc_full[h][buf]);
       }
+      // no commit arrives after the CTA has left: the last one covers every MMA of this thread
+      tc_commit(&bars->drain);
+      mbar_wait(&bars->drain, 0, kWaitLimitNs / 4);
     }
   } else {
     // ------------------------------------------------------------ epilogue
-    constexpr int HH = 1;                             // heads per epilogue warpgroup
-    const int ew = warp - 2;
+    const int wg = (warp - 2) >> 2;                   // heads wg, wg + kGroups, ..
     const int quad = warp & 3;                        // TMEM lanes 32 * (warp % 4) ..
-    const int hg = ew >> 2;                           // heads hg * HH ..
     const int kt = quad * 32 + lane;                  // key within the tile
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    float m[HH][kTcRows], sum[HH][kTcRows];
-#pragma unroll
-    for (int h = 0; h < HH; ++h)
-#pragma unroll
-      for (int j = 0; j < kTcRows; ++j) {
-        m[h][j] = -INFINITY;
-        sum[h][j] = 0.f;
-      }
     const float c2 = plan.scale2;
-    // modality of this thread's key, one tile ahead
-    uint8_t mod_next = (tb + kt < te) ? modality[sq.t0 + tb + kt] : 0;
-    for (int t = 0; t < ntiles; ++t) {
-      const int buf = t & 1;
-      const int key = tb + t * kTcM + kt;
-      const bool valid = key < te;
+    constexpr int kLanes = 32 / NR;                   // lanes per row after the reduce-scatter
+    int n = (wg - u0 % Lay::kGroups + Lay::kGroups) % Lay::kGroups;   // this warpgroup's stages: every kGroups-th
+    auto key_of = [&](int nn) { return ((u0 + nn) / HKV) * kTcM + kt; };
+    auto mod_of = [&](int nn) -> uint8_t {
+      const int key = key_of(nn);
+      return (nn < nstage && key < sq.len) ? modality[sq.t0 + key] : static_cast<uint8_t>(0);
+    };
+    uint8_t mod_next = mod_of(n);                     // one stage ahead
+    for (; n < nstage; n += Lay::kGroups) {
+      const int h = (u0 + n) % HKV, i = n / HKV, buf = i & 1;
+      const int key = key_of(n);
+      const bool valid = key < sq.len;
       const bool mm = valid && is_mm_tc(mod_next);
-      if (t + 1 < ntiles) mod_next = (key + kTcM < te) ? modality[sq.t0 + key + kTcM] : 0;
+      mod_next = mod_of(n + Lay::kGroups);
+      // rows j >= j_min have this key in their denominator: every row of a multimodal key, or
+      // (causal rows) the rows of the tokens at or after the key, token j / G >= key - q_pos
+      const int j_min = plan.causal ? (valid ? max(0, key - sq.q_pos) * G : NR) : (mm ? 0 : NR);
       // warp-uniform: tcgen05.ld below is a warp-collective instruction
-      if (!__all_sync(0xffffffffu, tc_wait(&bars->acc_full[buf], (t >> 1) & 1u, bars, err, 84))) break;
+      if (!__all_sync(0xffffffffu, tc_wait(&bars->acc_full[h][buf], (i >> 1) & 1u, bars, err, 84))) break;
       tc_fence_after();
-      uint32_t r[HH * kTcN];
-      const uint32_t taddr = bars->tmem_base + lane_off + buf * HKV * kTcN + hg * HH * kTcN;
-      tmem_ld16(taddr, r);
-      tmem_wait16(r);
+      uint32_t r[NR];
+      load_rows(bars->tmem_base + lane_off + (buf * HKV + h) * kN, r);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->acc_empty[buf]);   // the values are in registers
+      if (lane == 0) mbar_arrive(&bars->acc_empty[h][buf]);   // the values are in registers
+      float v[NR];
+      float *lp = logits + sq.logit_base + static_cast<int64_t>(h * G) * sq.lstride + key;
 #pragma unroll
-      for (int hh = 0; hh < HH; ++hh)
+      for (int j = 0; j < NR; ++j) {
+        const float x = __uint_as_float(r[j]);
+        if (valid && j < rg) lp[rho_of[j] * sq.lstride] = x;
+        v[j] = (j < rg && j >= j_min) ? x : -INFINITY;
+      }
+      // the row maxima of the warp's keys, then sums relative to the raised maxima
+      const int hh = Lay::kHeads == 1 ? 0 : h / Lay::kGroups;
+      const float tmax = reduce_scatter<NR>(v, lane, [](float a, float b) { return fmaxf(a, b); });
+      float m_old = m_run[0], l_old = l_run[0];
+      if (Lay::kHeads > 1 && hh) {
+        m_old = m_run[Lay::kHeads - 1];
+        l_old = l_run[Lay::kHeads - 1];
+      }
+      const float m_new = fmaxf(m_old, tmax * c2);    // log2 units; -inf while no key has counted
 #pragma unroll
-        for (int j = 0; j < kTcRows; ++j) {
-          if (j >= rg) continue;
-          const int h = hg * HH + hh;
-          const float y = __uint_as_float(r[hh * kTcN + j]) * c2;
-          const int rho = (j / G) * plan.hq + h * G + j % G;
-          if (valid) logits[sq.logit_base + static_cast<int64_t>(rho) * sq.lstride + key] = y;
-          // the row's denominator: multimodal keys, or (causal rows) every key up to its position
-          if (plan.causal ? (valid && key <= sq.q_pos + j / G) : mm) {
-            const float mn = fmaxf(m[hh][j], y);
-            sum[hh][j] = sum[hh][j] * ex2_approx(m[hh][j] - mn) + ex2_approx(y - mn);
-            m[hh][j] = mn;
-          }
-        }
-    }
-    // per-thread states into the (drained) ring after everyone is done, below
-    tc_fence_before();
-    __syncthreads();
-    if (!bars->abort) {
-      float2 *red = reinterpret_cast<float2 *>(ring);   // [128 keys][HKV * 8]
-#pragma unroll
-      for (int hh = 0; hh < HH; ++hh)
-#pragma unroll
-        for (int j = 0; j < kTcRows; ++j)
-          red[kt * (HKV * kTcRows) + (hg * HH + hh) * kTcRows + j] = make_float2(m[hh][j], sum[hh][j]);
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(tc_epi_warps<HKV>() * 32) : "memory");
-    if (!bars->abort) {
-      // one warp per (head, row): each lane folds 4 of the 128 per-key states, then a fixed
-      // shuffle tree combines the lanes (deterministic order)
-      const float2 *red = reinterpret_cast<const float2 *>(ring);
-      for (int e = ew; e < HKV * kTcRows; e += tc_epi_warps<HKV>()) {
-        const int h = e / kTcRows, j = e % kTcRows;
-        if (j >= rg) continue;                          // uniform over the warp
-        float2 v[kTcM / 32];
-        float mx = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < kTcM / 32; ++i) {
-          v[i] = red[(lane + 32 * i) * (HKV * kTcRows) + e];
-          mx = fmaxf(mx, v[i].x);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        float tot = 0.f;
-        if (mx != -INFINITY)
-#pragma unroll
-          for (int i = 0; i < kTcM / 32; ++i)
-            if (v[i].x != -INFINITY) tot += v[i].y * ex2_approx(v[i].x - mx);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
-        if (lane == 0) {
-          const int rho = (j / G) * plan.hq + h * G + j % G;
-          part[sq.part_base + static_cast<int64_t>(c - sq.unit8_begin) * sq.rows + rho] = make_float2(mx, tot);
-        }
+      for (int j = 0; j < NR; ++j) {
+        const float mj = __shfl_sync(0xffffffffu, m_new, j * kLanes);
+        // no counted key of the row yet: every term is exp2(-inf - 0) = 0
+        const float x = (j < rg && j >= j_min) ? __uint_as_float(r[j]) : -INFINITY;
+        v[j] = ex2_approx(fmaf(x, c2, mj == -INFINITY ? 0.f : -mj));
+      }
+      const float tsum = reduce_scatter<NR>(v, lane, [](float a, float b) { return a + b; });
+      const float l_new = (m_old == -INFINITY ? 0.f : l_old * ex2_approx(m_old - m_new)) + tsum;
+      if (Lay::kHeads > 1 && hh) {
+        m_run[Lay::kHeads - 1] = m_new;
+        l_run[Lay::kHeads - 1] = l_new;
+      } else {
+        m_run[0] = m_new;
+        l_run[0] = l_new;
       }
     }
-    // teardown below
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp == 1) tmem_dealloc(bars->tmem_base, Lay::kTmemCols);
-    return;
   }
-  // producer and MMA warps: after an abort make sure no MMA is in flight, then meet the
-  // epilogue at its two CTA barriers and free TMEM
-  if (warp == 1 && lane == 0 && bars->abort) {
-    tc_commit(&bars->drain);
-    mbar_wait(&bars->drain, 0, kWaitLimitNs / 4);
-  }
+  // every stage is consumed (or a wait gave up): the ring holds the warps' states next
   tc_fence_before();
   __syncthreads();
-  __syncthreads();
   tc_fence_after();
+  const bool ok = !bars->abort;
+  float2 *st = reinterpret_cast<float2 *>(ring);                        // [HKV][4 quads][NR]
+  if (ok && warp >= 2 && lane % (32 / NR) == 0) {
+    const int wg = (warp - 2) >> 2, quad = warp & 3;
+#pragma unroll
+    for (int i = 0; i < Lay::kHeads; ++i)
+      st[((wg + i * Lay::kGroups) * 4 + quad) * NR + lane / (32 / NR)] = make_float2(m_run[i], l_run[i]);
+  }
+  __syncthreads();
+  if (ok) {
+    for (int e = threadIdx.x; e < HKV * NR; e += Lay::kThreads) {
+      const int h = e / NR, j = e % NR;
+      if (j >= rg) continue;
+      float2 w[4];
+      float mx = -INFINITY, tot = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        w[i] = st[(h * 4 + i) * NR + j];
+        mx = fmaxf(mx, w[i].x);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (w[i].x != -INFINITY) tot += w[i].y * ex2_approx(w[i].x - mx);
+      part[sq.part_base + static_cast<int64_t>(rho_of[j] + h * G) * sq.nparts + c] = make_float2(mx, tot);
+    }
+  }
   if (warp == 1) tmem_dealloc(bars->tmem_base, Lay::kTmemCols);
+}
+
+template <int HKV, int NR>
+cudaError_t launch(int grid, cudaStream_t stream, const CUtensorMap &kmap, const NarrowPlan &P, const uint16_t *q,
+                   const uint8_t *modality, float *logits, float2 *part, DeviceError *err) {
+  using Lay = TcLayout<HKV, NR>;
+  static std::atomic<uint64_t> attr{0};
+  const cudaError_t e = once_per_device(attr, [] {
+    return cudaFuncSetAttribute(score_narrow_tc_kernel<HKV, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(Lay::kBytes));
+  });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(score_narrow_tc_kernel<HKV, NR>, dim3(grid), dim3(Lay::kThreads), Lay::kBytes, stream, kmap, P, q,
+                    modality, logits, part, err);
+}
+
+template <int HKV>
+cudaError_t launch_rows(int max_rg, int grid, cudaStream_t stream, const CUtensorMap &kmap, const NarrowPlan &P,
+                        const uint16_t *q, const uint8_t *modality, float *logits, float2 *part, DeviceError *err) {
+  if (max_rg <= 8) return launch<HKV, 8>(grid, stream, kmap, P, q, modality, logits, part, err);
+  if (max_rg <= 16) return launch<HKV, 16>(grid, stream, kmap, P, q, modality, logits, part, err);
+  return launch<HKV, 32>(grid, stream, kmap, P, q, modality, logits, part, err);
 }
 
 }  // namespace
 
-// Launches the tensor-core logits kernel for Hkv = 2 or 4 and at most 8 rows per head group.
-cudaError_t launch_narrow_tc(int grid, cudaStream_t stream, const CUtensorMap &kmap, const NarrowPlan &P,
+cudaError_t launch_narrow_tc(int max_rg, int grid, cudaStream_t stream, const CUtensorMap &kmap, const NarrowPlan &P,
                              const uint16_t *q, const uint8_t *modality, float *logits, float2 *part,
                              DeviceError *err) {
-  if (P.hkv == 4) {
-    static std::atomic<uint64_t> attr{0};
-    const cudaError_t e = once_per_device(attr, [] {
-      return cudaFuncSetAttribute(score_narrow_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(TcLayout<4>::kBytes));
-    });
-    if (e != cudaSuccess) return e;
-    return launch_pdl(score_narrow_tc_kernel<4>, dim3(grid), dim3(tc_threads<4>()), TcLayout<4>::kBytes, stream,
-                      kmap, P, q, modality, logits, part, err);
-  } else {
-    static std::atomic<uint64_t> attr{0};
-    const cudaError_t e = once_per_device(attr, [] {
-      return cudaFuncSetAttribute(score_narrow_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(TcLayout<2>::kBytes));
-    });
-    if (e != cudaSuccess) return e;
-    return launch_pdl(score_narrow_tc_kernel<2>, dim3(grid), dim3(tc_threads<2>()), TcLayout<2>::kBytes, stream,
-                      kmap, P, q, modality, logits, part, err);
+  switch (P.hkv) {
+    case 1: return launch_rows<1>(max_rg, grid, stream, kmap, P, q, modality, logits, part, err);
+    case 2: return launch_rows<2>(max_rg, grid, stream, kmap, P, q, modality, logits, part, err);
+    case 4: return launch_rows<4>(max_rg, grid, stream, kmap, P, q, modality, logits, part, err);
+    case 8: return launch_rows<8>(max_rg, grid, stream, kmap, P, q, modality, logits, part, err);
+    default: return cudaErrorInvalidValue;
   }
 }
 

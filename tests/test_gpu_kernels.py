@@ -113,6 +113,22 @@ def test_narrow_path_scores_match_oracle(ap, lens, nqs, hq, hkv):
     assert got.tobytes() == again.tobytes()
 
 
+@pytest.mark.parametrize("domain", [0, 1])
+@pytest.mark.parametrize("hq,hkv,nq", [(8, 1, 1), (8, 1, 2), (8, 1, 4), (16, 2, 4), (28, 4, 2), (28, 4, 4), (8, 8, 32),
+                                       (32, 8, 1), (32, 8, 3), (64, 8, 4), (12, 3, 3)])
+def test_narrow_path_head_layouts_and_row_counts(ap, hq, hkv, nq, domain):
+    """Every KV head count of the tensor-core kernel with 8, 16 and 32 rows per head group (and one
+    layout it does not take), tiles of one key, a key short of and past a tile, and a sequence cut
+    over many CTAs.  An fp32 dot product of 128 terms is off by at most 128 2^-24 sum|q k| = 1e-3
+    here, 1.3e-4 in the log2 logit; the normaliser's keys share the same bound."""
+    lens = [max(nq, 1), 127, 128, 129, 6401]
+    rng = np.random.default_rng(hq * 1000 + hkv * 100 + nq)
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, [nq] * len(lens), hq, hkv, scale_k=1.5)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
+    check_scores(got, ref, strict_rel=2e-4)
+
+
 def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap):
     """The general logits kernel writes one partial per 256 keys.  A batch of more than 256 keys per
     SM (38,912 tokens on 152 SMs) is one where a sequence has more of those than the tensor-core
