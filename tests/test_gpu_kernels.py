@@ -372,6 +372,48 @@ def test_select_matches_oracle_exactly(ap, lens, kind, mode):
     np.testing.assert_array_equal(ncu, oracle.new_cu_seqlens(ref, cu))
 
 
+def select_scores(rng, T, kind):
+    if kind == "lognormal":
+        return (np.exp(1.3 * rng.standard_normal(T)) / T).astype(np.float32)
+    if kind == "narrow":                    # thousands of scores in the k-th one's first bin
+        return (1e-5 * (1 + 1e-5 * rng.standard_normal(T)) + (rng.random(T) < 0.02)).astype(np.float32)
+    if kind == "wide":                      # 2^-126 .. 2^100, zeros and denormals: below the first level's binades
+        s = np.ldexp(rng.random(T), rng.integers(-140, 100, T)).astype(np.float32)
+        s[rng.random(T) < 0.2] = 0.0
+        return s
+    if kind == "two":                       # two values: every token ties
+        return np.where(rng.random(T) < 0.5, np.float32(0.25), np.float32(0.5))
+    return np.zeros(T, np.float32)          # one value
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("kind", ["lognormal", "narrow", "wide", "two", "zeros"])
+@pytest.mark.parametrize("lens", [
+    [1, 31, 32, 33, 1023, 1024, 1025],      # one CTA per sequence: rounds of 32 and 1,024 tokens and their neighbours
+    [9000, 0, 16383],                       # clusters of 4
+    [40001],                                # 8
+    [150000],                               # 16
+    [36864 * 16 + 5],                       # slices past the shared-memory copy
+])
+def test_select_score_distributions(ap, lens, kind, mode):
+    rng = np.random.default_rng(sum(lens) + mode)
+    mod = np.concatenate([rng.choice([0, 1, 2, 255], L, p=[0.04, 0.2, 0.75, 0.01]).astype(np.uint8) for L in lens])
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    sc = select_scores(rng, mod.size, kind)
+    na = [int((mod[cu[s]:cu[s + 1]] == 1).sum()) for s in range(len(lens))]
+    nv = [int((mod[cu[s]:cu[s + 1]] == 2).sum()) for s in range(len(lens))]
+    for frac in (0.0, 0.31, 1.0):
+        counts = [(int(frac * a), int(frac * v)) if mode == 0 else (int(frac * (a + v)), 0) for a, v in zip(na, nv)]
+        keep, mod_o, d2s, ncu, err = gpu_select(ap, sc, mod, cu, counts, na, nv, mode)
+        assert err == ap.APACK_OK
+        ref = oracle.select_keep(sc, mod, cu, counts, joint=True) if mode else oracle.select_keep(sc, mod, cu, counts)
+        np.testing.assert_array_equal(keep, ref)
+        np.testing.assert_array_equal(mod_o, mod[ref])
+        want = np.full(mod.size, -1, np.int32)
+        want[ref] = np.arange(ref.size)
+        np.testing.assert_array_equal(d2s, want)
+
+
 def test_select_reports_count_mismatch_without_faulting(ap):
     rng = np.random.default_rng(2)
     mod = rng.choice([0, 1, 2], 5000).astype(np.uint8)
