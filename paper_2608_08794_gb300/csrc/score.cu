@@ -60,8 +60,15 @@ constexpr int kCols = 64;                        // columns per TMEM load, pass 
 constexpr int kCols2 = 32;                       // columns per TMEM load, pass 2
 static_assert(2 * kSpan == 256 && 2 * kCols == kSpan && 4 * kCols2 == kSpan,
               "two warpgroups x (two or four) loads cover a 256-column tile");
-// warp 0: TMA, warp 1: TMEM (+ MMA on the even CTA), then the epilogue warps, then (pass 1) the
-// key-mask warp.  Nineteen warps take the same registers per thread as eighteen.
+// The epilogue bounds both passes, not the MMA: 64 columns loaded and summed by 16 warps take 1,220
+// clocks a tile (the exp2 unit 1,024, TMEM loads do not overlap it) against 1,024 for the MMA, and what
+// a warp does around its tiles comes on top, since the four warps of a scheduler tend to do it at the
+// same time.  So the loops run over a warpgroup's own tiles only, the masks come in one load, and the
+// exponentials are scheduled by hand (exp_sum): pass 1 188 -> 173 us, pass 2 170 -> 162 us over
+// 135,272 keys and 7,168 rows.  Measured slower: 8 epilogue warps with 64 or 128 columns in registers
+// (209 / 178 and 258 / 185 us), all 16 warps on every tile (197 / 187), half tiles of 128 columns
+// as MMAs of their own (200 / 206: N = 128 re-reads A from shared memory).
+// warp 0: TMA, warp 1: TMEM (+ MMA on the even CTA), then the epilogue warps.
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr uint32_t kTmemCols = 512;    // 2 accumulators x 256 fp32 columns
 constexpr int kAStages = 2, kBStages = 4;
@@ -233,9 +240,6 @@ __device__ __forceinline__ bool smem_aligned(const uint8_t *smem) { return (smem
 __device__ PairCtx init_pair(uint8_t *smem, Bars *bars, int warp) {
   PairCtx pc;
   pc.rank = cluster_ctarank();
-  // Zero the operand buffers once (every tile is then fully written by its TMA boxes).
-  for (uint32_t i = threadIdx.x; i < kOffL / 16; i += blockDim.x)
-    reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kAStages; ++i) {
       mbar_init(&bars->a_full[i], 1);
@@ -257,7 +261,6 @@ __device__ PairCtx init_pair(uint8_t *smem, Bars *bars, int warp) {
     bars->abort = 0;
     fence_mbar_init();
   }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   pc.lead_bars = map_shared_rank(bars, 0);
   pc.peer_abort = map_shared_rank(const_cast<const int32_t *>(&bars->abort), pc.rank ^ 1u);
   cluster_sync();                      // both CTAs' barriers exist before any remote arrive or copy
@@ -308,10 +311,11 @@ __device__ __forceinline__ void tmem_load_cols(uint32_t taddr, uint32_t (&r)[32]
 
 // The eight K=16 steps of one 256 x 256 x 128 product into accumulator `ci`.
 __device__ __forceinline__ void issue_mma(uint32_t tmem, int ci, uint32_t a_base, uint32_t b_base) {
+  const uint64_t a_desc = smem_desc_sw128(a_base), b_desc = smem_desc_sw128(b_base);
 #pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const uint32_t off = (kk >> 2) * kHalf + (kk & 3) * 32;
-    mma_pair(tmem + ci * 256, smem_desc_sw128(a_base + off), smem_desc_sw128(b_base + off), kk > 0 ? 1u : 0u);
+  for (int kk = 0; kk < 8; ++kk) {   // the address field counts 16 bytes; the tiles lie below 256 KB
+    const uint32_t off = ((kk >> 2) * kHalf + (kk & 3) * 32) >> 4;
+    mma_pair(tmem + ci * 256, a_desc + off, b_desc + off, kk > 0 ? 1u : 0u);
   }
 }
 
@@ -356,6 +360,42 @@ __device__ __forceinline__ Run next_run(const ScorePlan &p, int x, int x_end, in
 // partial sums keep the add chains short.
 constexpr float kSumLimit = 6.338253e29f;   // 2^99
 
+// a[0..3] += 2^(x c2 + add) over the N logits x of a thread, add(i) for logits i and i + 1; x is
+// overwritten.  The three steps of a group of kGroup logits (scale, exp2, sum) are written one group
+// apart and in place: the exp2 unit's latency is covered without registers for its results.
+constexpr int kGroup = 16;
+
+template <int N, class Add>
+__device__ __forceinline__ void exp_sum(uint32_t (&x)[N], float c2, Add add, float2 (&a)[4]) {
+  const float2 cc = make_float2(c2, c2);
+#pragma unroll
+  for (int g = 0; g < N / kGroup + 2; ++g) {
+    if (g >= 2) {
+#pragma unroll
+      for (int j = 0; j < kGroup; j += 2) {
+        const int i = (g - 2) * kGroup + j;
+        a[(i >> 1) & 3] = fadd2(a[(i >> 1) & 3], make_float2(__uint_as_float(x[i]), __uint_as_float(x[i + 1])));
+      }
+    }
+    if (g >= 1 && g - 1 < N / kGroup) {
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) {
+        const int i = (g - 1) * kGroup + j;
+        x[i] = __float_as_uint(ex2_approx(__uint_as_float(x[i])));
+      }
+    }
+    if (g < N / kGroup) {
+#pragma unroll
+      for (int j = 0; j < kGroup; j += 2) {
+        const int i = g * kGroup + j;
+        const float2 y = ffma2(make_float2(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), cc, add(i));
+        x[i] = __float_as_uint(y.x);
+        x[i + 1] = __float_as_uint(y.y);
+      }
+    }
+  }
+}
+
 __device__ __forceinline__ void online_block(uint32_t (&r)[64], uint32_t mask0, uint32_t mask1, float c2, float &m,
                                              float &sum, bool &bad) {
   if ((mask0 & mask1) != 0xffffffffu) {
@@ -374,12 +414,8 @@ __device__ __forceinline__ void online_block(uint32_t (&r)[64], uint32_t mask0, 
     m = mx * c2;
   }
   float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  const float2 cc = make_float2(c2, c2), nm = make_float2(-m, -m);
-#pragma unroll
-  for (int i = 0; i < 64; i += 2) {
-    const float2 y = ffma2(make_float2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), cc, nm);
-    a[(i >> 1) & 3] = fadd2(a[(i >> 1) & 3], make_float2(ex2_approx(y.x), ex2_approx(y.y)));
-  }
+  const float2 nm = make_float2(-m, -m);
+  exp_sum(r, c2, [&](int) { return nm; }, a);
   const float2 s01 = fadd2(a[0], a[1]), s23 = fadd2(a[2], a[3]);
   const float2 s4 = fadd2(s01, s23);
   const float t = s4.x + s4.y;
@@ -484,11 +520,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int quad = warp & 3;
     const int row = row_half + quad * 32 + lane;            // row of the 256-row pair
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const uint32_t acc_empty0 = lead_addr(pc, bars, &bars->acc_empty[0]);
+    const uint32_t acc_empty_own = lead_addr(pc, bars, &bars->acc_empty[own]);
+    const uint32_t tmem_q = bars->tmem_base + lane_off + own * 256 + col_base;
     const float c2 = plan.scale2;
     float2 *comb = reinterpret_cast<float2 *>(smem + kOffC);   // [2 parities][kEpiWG - 1 ranges][128 rows]
-    int ci = 0;
-    uint32_t cph = 0, xph = 0;
+    uint32_t tile0 = 0, cph = 0, xph = 0;                   // tiles of the runs before; own buffer's phase
     bool ok = true;
     for (int x = x_begin; ok && x < x_end;) {
       const Run w = next_run(plan, x, x_end, pair);
@@ -498,42 +534,39 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       bool bad = false;
       // causal rows: this lane's row (token r of the query span) sees keys up to q_pos + r
       const int see = sp.q_pos + (w.qp * kChunk + row) / G;
-      // the warpgroup's four 32-key mask words of a block (which keys count), one own block
-      // ahead: lane i < 4 holds word i, shuffled to every lane when the block is taken
-      const uint32_t *mwords = mask_words + sp.blk0 * 8 + (q & 1) * 4 + (lane & 3);
-      const int b_first = w.b0 + ((own - ci + 2) & 1);       // blocks alternate between the buffers
-      uint32_t m_next = (b_first < w.b1 && lane < 4) ? __ldg(mwords + b_first * 8) : 0u;
-      for (int b = w.b0; b < w.b1; ++b) {
-        if (ci == own) {
-          const uint32_t m_mine = m_next;
-          if (b + 2 < w.b1 && lane < 4) m_next = __ldg(mwords + (b + 2) * 8);
-          const uint4 mk = make_uint4(__shfl_sync(0xffffffffu, m_mine, 0), __shfl_sync(0xffffffffu, m_mine, 1),
-                                      __shfl_sync(0xffffffffu, m_mine, 2), __shfl_sync(0xffffffffu, m_mine, 3));
-          // the keys of this thread's words that count; and those this lane's row sees
-          uint32_t rm[4] = {mk.x, mk.y, mk.z, mk.w};
-          if (CAUSAL) {        // keys at local index <= see
+      // the warpgroup's four 32-key mask words of a block (which keys count), one own block ahead;
+      // the blocks alternate between the buffers
+      const uint4 *mwords = reinterpret_cast<const uint4 *>(mask_words + sp.blk0 * 8) + (q & 1);
+      const int b_first = w.b0 + ((own ^ tile0) & 1);
+      tile0 += w.b1 - w.b0;
+      uint4 m_next = b_first < w.b1 ? __ldg(mwords + b_first * 2) : make_uint4(0, 0, 0, 0);
+      for (int b = b_first; b < w.b1; b += 2) {
+        const uint4 mk = m_next;
+        if (b + 2 < w.b1) m_next = __ldg(mwords + (b + 2) * 2);
+        // the keys of this thread's words that count; and those this lane's row sees
+        uint32_t rm[4] = {mk.x, mk.y, mk.z, mk.w};
+        if (CAUSAL) {          // keys at local index <= see
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int lim = see - (b * kBlock + col_base + 32 * i);
-              rm[i] &= lim >= 31 ? 0xffffffffu : (lim < 0 ? 0u : (2u << lim) - 1u);
-            }
-          }
-          if (!wait_or_abort(&bars->acc_full[ci], cph, bars, pc, err, 16)) { ok = false; break; }
-          tc_fence_after();
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const bool any = (h == 0 ? (mk.x | mk.y) : (mk.z | mk.w)) != 0u;   // uniform over the warp
-            uint32_t rr[kCols];
-            if (any) tmem_load_cols(bars->tmem_base + lane_off + ci * 256 + col_base + h * kCols, rr);
-            if (h == 1) {     // both halves are in registers: release the buffer
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) arrive_cluster(acc_empty0 + ci * 8);
-            }
-            if (any) online_block(rr, rm[2 * h], rm[2 * h + 1], c2, m, sum, bad);
+          for (int i = 0; i < 4; ++i) {
+            const int lim = see - (b * kBlock + col_base + 32 * i);
+            rm[i] &= lim >= 31 ? 0xffffffffu : (lim < 0 ? 0u : (2u << lim) - 1u);
           }
         }
-        if (++ci == 2) { ci = 0; cph ^= 1; }
+        if (!wait_or_abort(&bars->acc_full[own], cph, bars, pc, err, 16)) { ok = false; break; }
+        cph ^= 1;
+        tc_fence_after();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool any = (h == 0 ? (mk.x | mk.y) : (mk.z | mk.w)) != 0u;   // uniform over the warp
+          uint32_t rr[kCols];
+          if (any) tmem_load_cols(tmem_q + h * kCols, rr);
+          if (h == 1) {     // both halves are in registers: release the buffer
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_cluster(acc_empty_own);
+          }
+          if (any) online_block(rr, rm[2 * h], rm[2 * h + 1], c2, m, sum, bad);
+        }
       }
       if (!ok) break;
       // the column ranges of each row combine in a fixed order (range 0 writes the pair's
@@ -690,7 +723,7 @@ __global__ void lse_merge_kernel(const __grid_constant__ ScorePlan plan, const f
       float dot = 0.f;
 #pragma unroll 16
       for (int d = 0; d < 128; ++d) dot = fmaf(qv[d], __uint_as_float(static_cast<uint32_t>(kr[d]) << 16), dot);
-      const float y = dot * plan.scale2;
+      const float y = dot * kScale2;                       // not from the tensor cores
       if (y > m) {
         sum = (m == -INFINITY ? 0.f : sum * exp2f(m - y)) + 1.f;
         m = y;
@@ -725,18 +758,9 @@ __device__ __forceinline__ Unit2 decode_unit2(const ScorePlan &p, int u) {
   return w;
 }
 
-// a[0..3] += 2^(x c2 + nl[col]) over the 32 columns of one load (four independent partial sums).
-__device__ __forceinline__ void colsum_word(const uint32_t (&r)[kCols2], const float *nl, float c2, float2 (&a)[4]) {
-  const float2 cc = make_float2(c2, c2);
-#pragma unroll
-  for (int i = 0; i < 32; i += 4) {
-    const float4 L = *reinterpret_cast<const float4 *>(nl + i);
-    const float2 y0 = ffma2(make_float2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), cc, make_float2(L.x, L.y));
-    const float2 y1 =
-        ffma2(make_float2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), cc, make_float2(L.z, L.w));
-    a[(i >> 2) & 3] = fadd2(a[(i >> 2) & 3], make_float2(ex2_approx(y0.x), ex2_approx(y0.y)));
-    a[(i >> 2) & 3] = fadd2(a[(i >> 2) & 3], make_float2(ex2_approx(y1.x), ex2_approx(y1.y)));
-  }
+// a[0..3] += 2^(x c2 + nl[col]) over the columns of one load (four independent partial sums).
+__device__ __forceinline__ void colsum_word(uint32_t (&r)[kCols2], const float *nl, float c2, float2 (&a)[4]) {
+  exp_sum(r, c2, [&](int i) { return *reinterpret_cast<const float2 *>(nl + i); }, a);
 }
 
 // The same over the columns i >= first only (causal rows that cannot see the key drop out;
@@ -856,11 +880,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int tkey = quad * 32 + lane;
     const int klane = row_half + tkey;                  // key of the 256-key unit
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const uint32_t acc_empty0 = lead_addr(pc, bars, &bars->acc_empty[0]);
+    const uint32_t acc_empty_own = lead_addr(pc, bars, &bars->acc_empty[own]);
+    const uint32_t tmem_q = bars->tmem_base + lane_off + own * 256 + col_base;
     const float c2 = plan.scale2;
     float *comb = reinterpret_cast<float *>(smem + kOffC);   // [2 parities][kEpiWG - 1 ranges][128 keys]
-    int ci = 0, li = 0;
-    uint32_t cph = 0, lph = 0, xph = 0;
+    uint32_t tile0 = 0, cph = 0, xph = 0;                   // chunks of the units before; own buffer's phase
     bool ok = true;
     for (int u = pair; ok && u < plan.total_units; u += npairs) {
       const Unit2 w = decode_unit2(plan, u);
@@ -870,49 +894,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
       // causal rows: only packed rows rho >= rho_min (tokens r >= key - q_pos) see this key
       const int rho_min = CAUSAL ? max(0, w.kp * kBlock + klane - sp.q_pos) * G : 0;
-      for (int c = 0; c < nch; ++c) {
-        if (ci == own) {   // chunks alternate between the buffers (normaliser slot li % 2 == ci)
-          if (!wait_or_abort(&bars->l_full[li], lph, bars, pc, err, 30)) { ok = false; break; }
-          if (!wait_or_abort(&bars->acc_full[ci], cph, bars, pc, err, 26)) { ok = false; break; }
-          tc_fence_after();
+      // chunks alternate between the buffers; normaliser slot = chunk % kBStages, an even number
+      const int c_first = (own ^ tile0) & 1;
+      for (int c = c_first; c < nch; c += 2) {
+        const uint32_t t = tile0 + c, li = t % kBStages;
+        if (!wait_or_abort(&bars->l_full[li], (t / kBStages) & 1, bars, pc, err, 30)) { ok = false; break; }
+        if (!wait_or_abort(&bars->acc_full[own], cph, bars, pc, err, 26)) { ok = false; break; }
+        cph ^= 1;
+        tc_fence_after();
 #pragma unroll
-          for (int h = 0; h < kSpan / kCols2; ++h) {
-            const int col0 = col_base + h * kCols2;
-            const float *nl = lse_s + li * kChunk + col0;
-            uint32_t rr[kCols2];
-            tmem_load_cols(bars->tmem_base + lane_off + ci * 256 + col0, rr);
-            if (h == kSpan / kCols2 - 1) {     // every column is in registers: release the buffer
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) arrive_cluster(acc_empty0 + ci * 8);
-            }
-            const int first = rho_min - (c * kChunk + col0);
-            if (!CAUSAL || first <= 0)
-              colsum_word(rr, nl, c2, a);
-            else if (first < kCols2)
-              colsum_word_from(rr, nl, c2, first, a);
+        for (int h = 0; h < kSpan / kCols2; ++h) {
+          const int col0 = col_base + h * kCols2;
+          const float *nl = lse_s + li * kChunk + col0;
+          uint32_t rr[kCols2];
+          tmem_load_cols(tmem_q + h * kCols2, rr);
+          if (h == kSpan / kCols2 - 1) {     // every column is in registers: release the buffer
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_cluster(acc_empty_own);
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bars->l_empty[li]);
+          const int first = rho_min - (c * kChunk + col0);
+          if (!CAUSAL || first <= 0)
+            colsum_word(rr, nl, c2, a);
+          else if (first < kCols2)
+            colsum_word_from(rr, nl, c2, first, a);
         }
-        if (++ci == 2) { ci = 0; cph ^= 1; }
-        if (++li == kBStages) { li = 0; lph ^= 1; }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->l_empty[li]);
       }
+      tile0 += nch;
       if (!ok) break;
       const float2 s01 = fadd2(a[0], a[1]), s23 = fadd2(a[2], a[3]);
       const float2 s4 = fadd2(s01, s23);
       const float mine = s4.x + s4.y;
       float *cb = comb + (xph & 1) * (kEpiWG - 1) * kRows;
-      if (q > 0) {
+      if (q < kEpiWG - 1) {
         if (!wait_or_abort(&bars->comb_empty[xph & 1], ((xph >> 1) & 1) ^ 1, bars, pc, err, 27)) break;
-        cb[(q - 1) * kRows + tkey] = mine;
+        cb[q * kRows + tkey] = mine;
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->comb_full[xph & 1]);
       } else {
         if (!wait_or_abort(&bars->comb_full[xph & 1], (xph >> 1) & 1, bars, pc, err, 28)) break;
-        float tot = mine;
+        float tot = cb[tkey];
 #pragma unroll
-        for (int i = 1; i < kEpiWG; ++i) tot += cb[(i - 1) * kRows + tkey];   // fixed order
+        for (int i = 1; i < kEpiWG - 1; ++i) tot += cb[i * kRows + tkey];   // fixed order
+        tot += mine;
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->comb_empty[xph & 1]);
         const int key = sp.t0 + w.kp * kBlock + klane;
@@ -1069,7 +1095,7 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
     P.group = G;
     P.total_qrows = static_cast<int32_t>(NQ);
     P.total_tokens = static_cast<int32_t>(T);
-    P.scale2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(APACK_HEAD_DIM)));
+    P.scale2 = kScale2Tc;
     P.causal = seqs->softmax_domain == APACK_SOFTMAX_CAUSAL_ROW;
     int64_t qrows = 0, flat = 0, nb_max = 0;
     int units2 = 0, blocks = 0;
