@@ -10,13 +10,16 @@
 //     exp2) over its keys.  The (row group, key block) space is cut into equal
 //     contiguous ranges, one per CTA pair; a pair writes one partial (m, sum) per
 //     row for each row group its range touches.
-//  merge: per packed query row, the partials combine into a log2-domain
+//  merge: per packed query row, the partials combine in pair order into a log2-domain
 //     normaliser lse2 = log2 sum_j 2^(x_j log2(e)/sqrt(D)), stored negated (a row whose
 //     logits overflowed its run's reference is recomputed there exactly).
 //  pass 2 (column sums): D[key][row] = K . Q^T with keys in TMEM lanes; each
 //     thread owns one key and sums 2^(x c - lse2[row]) over the rows of one KV
-//     head group; a final pass adds the Hkv group sums in a fixed order and
-//     scales by 1/(Hq n_q).  No atomics anywhere: scores are deterministic.
+//     head group; the Hkv group sums are added in a fixed order and scaled by
+//     1/(Hq n_q): by the unit itself when it runs over every group, else by the last
+//     unit of a key block (a counter), else (long sequences whose groups are better
+//     split, or sequences without query rows in the launch) by a final kernel.
+//     Scores are deterministic: the counters only say who adds, not in what order.
 //
 // Query rows are first repacked per KV head g into linear rows rho = token * G + j
 // (query head g*G + j), padded to a multiple of 256, so that tiles hold no holes.
@@ -35,8 +38,7 @@
 // blocks in pass 1, query chunks in pass 2), four B stages deep; two 256-column
 // accumulators alternate in TMEM.  Warp 0 issues TMA, warp 1 owns TMEM (and on the
 // even CTA issues the MMAs), warps 2..17 are four epilogue warpgroups; warpgroups 2b
-// and 2b + 1 read the tiles of accumulator b, 128 columns each for the CTA's 128 lanes,
-// in two TMEM loads of 64.  Pass 1 takes each key block's masks (which keys count)
+// and 2b + 1 read the tiles of accumulator b, 128 columns each for the CTA's 128 lanes.  Pass 1 takes each key block's masks (which keys count)
 // from a bit array that the query repack kernel writes once per call.  Operands sit in
 // 128-byte swizzled shared memory.  Persistent pairs, one CTA per SM.
 #include <cmath>
@@ -80,6 +82,8 @@ constexpr int kBlock = 256;                    // keys per key block (pass 1) / 
 constexpr int kChunk = 256;                    // query rows per chunk (pass 2) / per row pair (pass 1)
 constexpr int kPairSlots = kMaxSplits;         // pair ranges per row group (one partial each)
 
+constexpr int kMergeThreads = 64;
+
 struct SeqPlan {
   int32_t t0, len;        // token range of the sequence in the packed batch
   int32_t q_off, n_q;     // query tokens in packed Q
@@ -101,6 +105,9 @@ struct ScorePlan {
   int32_t total_qrows;     // sum n_q over the whole batch
   int32_t total_tokens;    // T
   int32_t causal;          // APACK_SOFTMAX_CAUSAL_ROW: rows see every token up to their own position
+  int32_t unit_groups;     // pass 2: KV head groups per unit, 1 or hkv
+  int32_t direct;          // pass 2: a unit holds every group and writes its keys' scores
+  int32_t counted;         // pass 2, one of several groups per unit: the last of a key block's units adds them
   float scale2;            // log2(e) / sqrt(D)
   SeqPlan seq[kSeqsPerLaunch];
 };
@@ -125,6 +132,12 @@ constexpr uint32_t kOffBars = kOffC + 2 * (kEpiWG - 1) * kRows * sizeof(float2);
 constexpr uint32_t kSmemBytes = kOffBars + 512;
 static_assert(sizeof(Bars) <= 512, "barrier block");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
+
+// pass 2 counters of a launch (one word per key block, 4 bits per 32 keys) in the workspace, where the
+// in-place compaction keeps its progress words later in the step
+constexpr size_t kCounterOff = 256;
+constexpr int kMaxCounted = 192;               // key blocks
+constexpr int kMaxCountedGroups = 15;          // what 4 bits count
 
 __device__ __forceinline__ bool is_mm(uint8_t m) { return m == APACK_MOD_AUDIO || m == APACK_MOD_VISUAL; }
 
@@ -428,7 +441,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     score_rowstats_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                           const __grid_constant__ ScorePlan plan, const uint32_t *__restrict__ mask_words,
                           float2 *__restrict__ part, DeviceError *err) {
-  pdl_wait_and_release();
   extern __shared__ __align__(1024) uint8_t smem[];
   if (!smem_aligned(smem)) {   // the same in both CTAs of the pair: both leave here
     if (threadIdx.x == 0) raise_device_error(err, APACK_EDEVICE, 10);
@@ -437,6 +449,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   Bars *bars = reinterpret_cast<Bars *>(smem + kOffBars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PairCtx pc = init_pair(smem, bars, warp);
+  pdl_wait_and_release();      // the set-up runs beside the previous launch
   const int G = plan.group;
   const int pair = blockIdx.x >> 1;
   const int x_begin = range_start(pair, plan.pairs, plan.flat_total);
@@ -621,7 +634,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 __global__ void q_pack_kernel(const __grid_constant__ ScorePlan plan, const uint4 *__restrict__ q,
                               uint4 *__restrict__ qp, int64_t row_begin, int64_t n_vec,
                               const uint8_t *__restrict__ modality, uint32_t *__restrict__ mask_words,
-                              int64_t n_words) {
+                              int64_t n_words, uint32_t *__restrict__ counters) {
   pdl_wait_and_release();
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (e >= n_vec) {
@@ -641,6 +654,7 @@ __global__ void q_pack_kernel(const __grid_constant__ ScorePlan plan, const uint
       if (key < t_end && (plan.causal || is_mm(modality[key]))) word |= 1u << k;
     }
     mask_words[wd] = word;
+    if (c == 0 && plan.counted) counters[gb] = 0u;       // pass 2's count of the block's finished units
     return;
   }
   const int64_t prow = row_begin + e / 16;
@@ -660,91 +674,107 @@ __global__ void q_pack_kernel(const __grid_constant__ ScorePlan plan, const uint
 }
 
 // ------------------------------------------------------------------ merge
-// One warp per packed query row (sequence, KV head group, rho); writes -lse2 at the row's
-// packed index (padding rows -inf, so that they add exp2(-inf) = 0).  Lane p takes the partial
-// of pair range p (at most 32), and a fixed shuffle tree combines them: deterministic.
-//
-// A row with a partial marked out of range (negative sum: a logit far above its run's
-// reference) is recomputed exactly here instead: the warp's lanes take every 32nd key of
-// the sequence, dot it with the row's query vector in fp32 from the bf16 values, keep an
-// online (max, sum of exp2) with exact rescaling, and combine in a fixed order.  Slow, and
-// only taken for inputs whose logits span more than about 99 binary orders of magnitude.
+// Negated log2 normaliser of one query row (token r of the span, packed row qr) of KV head group g,
+// computed by a warp without the tensor cores: the lanes take every 32nd key of the sequence, dot it
+// with the row in fp32 from the bf16 values, keep an online (max, sum of exp2) with exact rescaling, and
+// combine in a fixed order.  Slow, and only taken for inputs whose logits span more than about 99
+// binary orders of magnitude (a partial marked by a negative sum).
 template <bool CAUSAL>
-__global__ void lse_merge_kernel(const __grid_constant__ ScorePlan plan, const float2 *__restrict__ part,
-                                 const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k,
-                                 int64_t k_stride, const uint8_t *__restrict__ modality, float *__restrict__ nlse2,
-                                 int64_t row_begin, int64_t n_rows) {
+__device__ float exact_nlse(const SeqPlan &sp, int g, int r, const uint16_t *__restrict__ qr,
+                                         const uint8_t *__restrict__ k, int64_t k_stride,
+                                         const uint8_t *__restrict__ modality) {
+  const int see = sp.q_pos + r;                         // causal rows: keys up to the row's position
+  float m = -INFINITY, sum = 0.f;
+  for (int key = sp.t0 + (threadIdx.x & 31); key < sp.t0 + sp.len; key += 32) {
+    if (CAUSAL ? key - sp.t0 > see : !is_mm(modality[key])) continue;
+    const uint16_t *kr = reinterpret_cast<const uint16_t *>(k + key * k_stride) + g * 128;
+    float dot = 0.f;
+#pragma unroll 8
+    for (int d = 0; d < 128; ++d)
+      dot = fmaf(__uint_as_float(static_cast<uint32_t>(qr[d]) << 16), __uint_as_float(static_cast<uint32_t>(kr[d]) << 16),
+                 dot);
+    const float y = dot * kScale2;                      // not from the tensor cores
+    if (y > m) {
+      sum = (m == -INFINITY ? 0.f : sum * exp2f(m - y)) + 1.f;
+      m = y;
+    } else {
+      sum += exp2f(y - m);
+    }
+  }
+  float mm = m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+  float tot = (m != -INFINITY) ? sum * exp2f(m - mm) : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  return mm == -INFINITY ? INFINITY : -(mm + log2f(tot));
+}
+
+// One thread per packed query row (sequence, KV head group, rho); writes -lse2 at the row's packed index
+// (padding rows -inf, so that they add exp2(-inf) = 0).  The partials of the pair ranges that touched the
+// row group (at most 32) are taken in pair order, kBatch of them loaded together: deterministic.  Bound by
+// latency: one or two L2 round trips.  A warp per row, one partial per lane, took 25 us for 68,608 rows;
+// this takes 4.8 us.  A row with a partial marked out of range (negative sum) is recomputed exactly by
+// its warp.
+template <bool CAUSAL>
+__global__ void __launch_bounds__(kMergeThreads)
+    lse_merge_kernel(const __grid_constant__ ScorePlan plan, const float2 *__restrict__ part,
+                     const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k, int64_t k_stride,
+                     const uint8_t *__restrict__ modality, float *__restrict__ nlse2, int64_t row_begin) {
   pdl_wait_and_release();
-  __shared__ float qsh[8][128];                           // the query row of each warp (fallback only)
-  const int64_t e = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  if (e >= n_rows) return;
-  const int64_t prow = row_begin + e;
+  // the rows of a launch are a multiple of 256: whole CTAs, and a row group never ends inside a warp
+  const int64_t prow = row_begin + blockIdx.x * static_cast<int64_t>(kMergeThreads) + threadIdx.x;
   int s = 0;
   while (s + 1 < plan.nseq && plan.seq[s + 1].qp_base <= prow) ++s;
   const SeqPlan &sp = plan.seq[s];
   const int G = plan.group;
   const int local = static_cast<int>(prow - sp.qp_base);
   const int g = local / sp.rows_pad, rho = local - g * sp.rows_pad;
-  if (rho >= G * sp.n_q) {
-    if (lane == 0) nlse2[prow] = -INFINITY;
-    return;
-  }
+  const bool real = rho < G * sp.n_q;
   const int r = rho / G, j = rho - r * G;
-  const int qrow = sp.q_off + r;
-  const int h = g * G + j;
   // the pair ranges that touched this row group, one partial each
-  const int grp = g * n_pairs(sp) + rho / kChunk;
-  const int x0 = sp.flat0 + grp * sp.nb;
+  const int x0 = sp.flat0 + (g * n_pairs(sp) + rho / kChunk) * sp.nb;
   const int np = sp.nb > 0 ? pair_of(x0 + sp.nb - 1, plan.pairs, plan.flat_total) -
                                  pair_of(x0, plan.pairs, plan.flat_total) + 1
                            : 0;
-  float2 v = make_float2(-INFINITY, 0.f);
-  if (lane < np) v = part[(static_cast<size_t>(lane) * plan.total_qrows + qrow) * plan.hq + h];
-  float out;
-  if (__ballot_sync(0xffffffffu, v.y < 0.f) == 0u) {
-    float mm = v.x;
+  float out = -INFINITY;
+  bool exact = false;
+  if (real) {
+    const float2 *p = part + static_cast<size_t>(sp.q_off + r) * plan.hq + g * G + j;
+    const size_t stride = static_cast<size_t>(plan.total_qrows) * plan.hq;
+    float m = -INFINITY, tot = 0.f;
+    constexpr int kBatch = 8;
+    for (int i0 = 0; i0 < np; i0 += kBatch) {
+      float2 v[kBatch];
+      float mn = m;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-    float tot = (v.x != -INFINITY) ? v.y * exp2f(v.x - mm) : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    out = mm == -INFINITY ? INFINITY : -(mm + log2f(tot));   // no key at all (S empty): nothing is scored
-  } else {
-    float *qv = qsh[wib];
-    const uint16_t *qr = qp + prow * 128;
-    for (int d = lane; d < 128; d += 32) qv[d] = __uint_as_float(static_cast<uint32_t>(qr[d]) << 16);
-    __syncwarp();
-    const int see = sp.q_pos + r;                         // causal rows: keys up to the row's position
-    float m = -INFINITY, sum = 0.f;
-    for (int key = sp.t0 + lane; key < sp.t0 + sp.len; key += 32) {
-      if (CAUSAL ? key - sp.t0 > see : !is_mm(modality[key])) continue;
-      const uint16_t *kr = reinterpret_cast<const uint16_t *>(k + key * k_stride) + g * 128;
-      float dot = 0.f;
-#pragma unroll 16
-      for (int d = 0; d < 128; ++d) dot = fmaf(qv[d], __uint_as_float(static_cast<uint32_t>(kr[d]) << 16), dot);
-      const float y = dot * kScale2;                       // not from the tensor cores
-      if (y > m) {
-        sum = (m == -INFINITY ? 0.f : sum * exp2f(m - y)) + 1.f;
-        m = y;
-      } else {
-        sum += exp2f(y - m);
+      for (int i = 0; i < kBatch; ++i) {
+        v[i] = i0 + i < np ? p[(i0 + i) * stride] : make_float2(-INFINITY, 0.f);
+        mn = fmaxf(mn, v[i].x);
       }
+      if (m != -INFINITY) tot *= exp2f(m - mn);
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        exact |= v[i].y < 0.f;
+        if (v[i].x != -INFINITY) tot += v[i].y * exp2f(v[i].x - mn);
+      }
+      m = mn;
     }
-    float mm = m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-    float tot = (m != -INFINITY) ? sum * exp2f(m - mm) : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    out = mm == -INFINITY ? INFINITY : -(mm + log2f(tot));
+    out = m == -INFINITY ? INFINITY : -(m + log2f(tot));   // no key at all (S empty): nothing is scored
   }
-  if (lane == 0) nlse2[prow] = out;
+  const int lane = threadIdx.x & 31;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, exact); todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const float x = exact_nlse<CAUSAL>(sp, g, __shfl_sync(0xffffffffu, r, l), qp + (prow - lane + l) * 128, k, k_stride,
+                                       modality);
+    if (lane == l) out = x;
+  }
+  nlse2[prow] = out;
 }
 
 // ------------------------------------------------------------------ pass 2
 struct Unit2 {
-  int s, kp, g;
+  int s, kp, g;            // sequence, key block, first KV head group (plan.unit_groups of them)
 };
 
 __device__ __forceinline__ Unit2 decode_unit2(const ScorePlan &p, int u) {
@@ -753,8 +783,12 @@ __device__ __forceinline__ Unit2 decode_unit2(const ScorePlan &p, int u) {
   while (s + 1 < p.nseq && p.seq[s + 1].unit_begin <= u) ++s;
   w.s = s;
   const int local = u - p.seq[s].unit_begin;
-  w.g = local % p.hkv;
-  w.kp = local / p.hkv;
+  w.g = 0;
+  w.kp = local;
+  if (p.unit_groups == 1) {
+    w.kp = local / p.hkv;
+    w.g = local - w.kp * p.hkv;
+  }
   return w;
 }
 
@@ -772,14 +806,16 @@ __device__ __forceinline__ void colsum_word_from(const uint32_t (&r)[kCols2], co
     if (i >= first) a[i & 3].x += ex2_approx(fmaf(__uint_as_float(r[i]), c2, nl[i]));
 }
 
-// Work unit = (256 keys, KV head group g): 128 keys per CTA of the pair; writes the group's
-// sum for each key to gsum[g][key]; the final kernel adds the groups.
+// Work unit = (256 keys, KV head group g) or (256 keys, every group): 128 keys per CTA of the pair.
+// A unit of every group writes its keys' scores.  A unit of one group writes the group's sums to
+// gsum[g][key]; with counters the last of a key block's units then adds the groups (every warp for its
+// 32 keys), without them the final kernel does.
 template <bool CAUSAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     score_colsum_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
-                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2,
-                        float *__restrict__ gsum, DeviceError *err) {
-  pdl_wait_and_release();
+                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2, float *gsum,
+                        uint32_t *counters, const uint8_t *__restrict__ modality, float *__restrict__ scores,
+                        DeviceError *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   if (!smem_aligned(smem)) {   // the same in both CTAs of the pair: both leave here
     if (threadIdx.x == 0) raise_device_error(err, APACK_EDEVICE, 10);
@@ -789,6 +825,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   float *lse_s = reinterpret_cast<float *>(smem + kOffL);   // [4][256], indexed by B stage
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PairCtx pc = init_pair(smem, bars, warp);
+  pdl_wait_and_release();      // the set-up runs beside the previous launch
   const int G = plan.group;
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const int row_half = static_cast<int>(pc.rank) * kRows;   // this CTA's keys of a unit, rows of a chunk
@@ -807,32 +844,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const SeqPlan &sp = plan.seq[w.s];
         const int nch = sp.rows_pad / kChunk;
         if (nch == 0) continue;
-        if (!wait_or_abort(&bars->a_empty[ai], aph ^ 1, bars, pc, err, 21)) { ok = false; break; }
-        uint8_t *A = smem + kOffA + ai * kTileBytes;
-        if (pc.rank == 0) mbar_arrive_expect_tx(&bars->a_full[ai], 2 * kTileBytes);
-        const uint32_t afull = lead_addr(pc, bars, &bars->a_full[ai]);
-        const int key0 = sp.t0 + w.kp * kBlock + row_half;
-        tma_load_3d_pair(A, &kmap, afull, 0, w.g, key0);
-        tma_load_3d_pair(A + kHalf, &kmap, afull, 64, w.g, key0);
-        apend[ai] = true;
-        apend_par[ai] = aph;
-        for (int c = 0; c < nch; ++c) {
-          if (!wait_or_abort(&bars->b_empty[bi], bph ^ 1, bars, pc, err, 22)) { ok = false; break; }
-          // normaliser slot bi is free once this CTA's epilogue of the chunk that used it is done
-          if (!wait_or_abort(&bars->l_empty[bi], bph ^ 1, bars, pc, err, 29)) { ok = false; break; }
-          const int64_t row0 = static_cast<int64_t>(sp.qp_base) + w.g * sp.rows_pad + c * kChunk;
-          mbar_arrive_expect_tx(&bars->l_full[bi], kChunk * sizeof(float));
-          bulk_load(lse_s + bi * kChunk, nlse2 + row0, kChunk * sizeof(float), &bars->l_full[bi]);
-          uint8_t *B = smem + kOffB + bi * kTileBytes;
-          if (pc.rank == 0) mbar_arrive_expect_tx(&bars->b_full[bi], 2 * kTileBytes);
-          const uint32_t bfull = lead_addr(pc, bars, &bars->b_full[bi]);
-          tma_load_3d_pair(B, &qmap, bfull, 0, 0, static_cast<int32_t>(row0) + row_half);
-          tma_load_3d_pair(B + kHalf, &qmap, bfull, 64, 0, static_cast<int32_t>(row0) + row_half);
-          pend[bi] = true;
-          pend_par[bi] = bph;
-          if (++bi == kBStages) { bi = 0; bph ^= 1; }
+        for (int g = w.g; ok && g < w.g + plan.unit_groups; ++g) {
+          if (!wait_or_abort(&bars->a_empty[ai], aph ^ 1, bars, pc, err, 21)) { ok = false; break; }
+          uint8_t *A = smem + kOffA + ai * kTileBytes;
+          if (pc.rank == 0) mbar_arrive_expect_tx(&bars->a_full[ai], 2 * kTileBytes);
+          const uint32_t afull = lead_addr(pc, bars, &bars->a_full[ai]);
+          const int key0 = sp.t0 + w.kp * kBlock + row_half;
+          tma_load_3d_pair(A, &kmap, afull, 0, g, key0);
+          tma_load_3d_pair(A + kHalf, &kmap, afull, 64, g, key0);
+          apend[ai] = true;
+          apend_par[ai] = aph;
+          for (int c = 0; c < nch; ++c) {
+            if (!wait_or_abort(&bars->b_empty[bi], bph ^ 1, bars, pc, err, 22)) { ok = false; break; }
+            // normaliser slot bi is free once this CTA's epilogue of the chunk that used it is done
+            if (!wait_or_abort(&bars->l_empty[bi], bph ^ 1, bars, pc, err, 29)) { ok = false; break; }
+            const int64_t row0 = static_cast<int64_t>(sp.qp_base) + g * sp.rows_pad + c * kChunk;
+            mbar_arrive_expect_tx(&bars->l_full[bi], kChunk * sizeof(float));
+            bulk_load(lse_s + bi * kChunk, nlse2 + row0, kChunk * sizeof(float), &bars->l_full[bi]);
+            uint8_t *B = smem + kOffB + bi * kTileBytes;
+            if (pc.rank == 0) mbar_arrive_expect_tx(&bars->b_full[bi], 2 * kTileBytes);
+            const uint32_t bfull = lead_addr(pc, bars, &bars->b_full[bi]);
+            tma_load_3d_pair(B, &qmap, bfull, 0, 0, static_cast<int32_t>(row0) + row_half);
+            tma_load_3d_pair(B + kHalf, &qmap, bfull, 64, 0, static_cast<int32_t>(row0) + row_half);
+            pend[bi] = true;
+            pend_par[bi] = bph;
+            if (++bi == kBStages) { bi = 0; bph ^= 1; }
+          }
+          if (++ai == kAStages) { ai = 0; aph ^= 1; }
         }
-        if (++ai == kAStages) { ai = 0; aph ^= 1; }
       }
       if (!ok) {
         // this CTA's normaliser copies complete on its own barriers
@@ -853,21 +892,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const Unit2 w = decode_unit2(plan, u);
         const int nch = plan.seq[w.s].rows_pad / kChunk;
         if (nch == 0) continue;
-        if (!wait_or_abort(&bars->a_full[ai], aph, bars, pc, err, 23)) { ok = false; break; }
-        const uint32_t a_base = smem_u32(smem + kOffA + ai * kTileBytes);
-        for (int c = 0; c < nch; ++c) {
-          if (!wait_or_abort(&bars->b_full[bi], bph, bars, pc, err, 24)) { ok = false; break; }
-          if (!wait_or_abort(&bars->acc_empty[ci], cph ^ 1, bars, pc, err, 25)) { ok = false; break; }
-          tc_fence_after();
-          issue_mma(tmem, ci, a_base, smem_u32(smem + kOffB + bi * kTileBytes));
-          commit_pair(&bars->b_empty[bi]);
-          commit_pair(&bars->acc_full[ci]);
-          if (++bi == kBStages) { bi = 0; bph ^= 1; }
-          if (++ci == 2) { ci = 0; cph ^= 1; }
+        for (int g = 0; ok && g < plan.unit_groups; ++g) {
+          if (!wait_or_abort(&bars->a_full[ai], aph, bars, pc, err, 23)) { ok = false; break; }
+          const uint32_t a_base = smem_u32(smem + kOffA + ai * kTileBytes);
+          for (int c = 0; c < nch; ++c) {
+            if (!wait_or_abort(&bars->b_full[bi], bph, bars, pc, err, 24)) { ok = false; break; }
+            if (!wait_or_abort(&bars->acc_empty[ci], cph ^ 1, bars, pc, err, 25)) { ok = false; break; }
+            tc_fence_after();
+            issue_mma(tmem, ci, a_base, smem_u32(smem + kOffB + bi * kTileBytes));
+            commit_pair(&bars->b_empty[bi]);
+            commit_pair(&bars->acc_full[ci]);
+            if (++bi == kBStages) { bi = 0; bph ^= 1; }
+            if (++ci == 2) { ci = 0; cph ^= 1; }
+          }
+          if (!ok) break;
+          commit_pair(&bars->a_empty[ai]);
+          if (++ai == kAStages) { ai = 0; aph ^= 1; }
         }
-        if (!ok) break;
-        commit_pair(&bars->a_empty[ai]);
-        if (++ai == kAStages) { ai = 0; aph ^= 1; }
       }
     }
   } else {
@@ -891,42 +932,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const SeqPlan &sp = plan.seq[w.s];
       const int nch = sp.rows_pad / kChunk;
       if (nch == 0) continue;
-      float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
       // causal rows: only packed rows rho >= rho_min (tokens r >= key - q_pos) see this key
       const int rho_min = CAUSAL ? max(0, w.kp * kBlock + klane - sp.q_pos) * G : 0;
-      // chunks alternate between the buffers; normaliser slot = chunk % kBStages, an even number
-      const int c_first = (own ^ tile0) & 1;
-      for (int c = c_first; c < nch; c += 2) {
-        const uint32_t t = tile0 + c, li = t % kBStages;
-        if (!wait_or_abort(&bars->l_full[li], (t / kBStages) & 1, bars, pc, err, 30)) { ok = false; break; }
-        if (!wait_or_abort(&bars->acc_full[own], cph, bars, pc, err, 26)) { ok = false; break; }
-        cph ^= 1;
-        tc_fence_after();
+      float mine = 0.f;                                     // the groups' sums, in group order
+      for (int g = 0; ok && g < plan.unit_groups; ++g) {
+        float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        // chunks alternate between the buffers; normaliser slot = chunk % kBStages, an even number
+        for (int c = (own ^ tile0) & 1; c < nch; c += 2) {
+          const uint32_t t = tile0 + c, li = t % kBStages;
+          if (!wait_or_abort(&bars->l_full[li], (t / kBStages) & 1, bars, pc, err, 30)) { ok = false; break; }
+          if (!wait_or_abort(&bars->acc_full[own], cph, bars, pc, err, 26)) { ok = false; break; }
+          cph ^= 1;
+          tc_fence_after();
 #pragma unroll
-        for (int h = 0; h < kSpan / kCols2; ++h) {
-          const int col0 = col_base + h * kCols2;
-          const float *nl = lse_s + li * kChunk + col0;
-          uint32_t rr[kCols2];
-          tmem_load_cols(tmem_q + h * kCols2, rr);
-          if (h == kSpan / kCols2 - 1) {     // every column is in registers: release the buffer
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_cluster(acc_empty_own);
+          for (int h = 0; h < kSpan / kCols2; ++h) {
+            const int col0 = col_base + h * kCols2;
+            const float *nl = lse_s + li * kChunk + col0;
+            uint32_t rr[kCols2];
+            tmem_load_cols(tmem_q + h * kCols2, rr);
+            if (h == kSpan / kCols2 - 1) {     // every column is in registers: release the buffer
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) arrive_cluster(acc_empty_own);
+            }
+            const int first = rho_min - (c * kChunk + col0);
+            if (!CAUSAL || first <= 0)
+              colsum_word(rr, nl, c2, a);
+            else if (first < kCols2)
+              colsum_word_from(rr, nl, c2, first, a);
           }
-          const int first = rho_min - (c * kChunk + col0);
-          if (!CAUSAL || first <= 0)
-            colsum_word(rr, nl, c2, a);
-          else if (first < kCols2)
-            colsum_word_from(rr, nl, c2, first, a);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->l_empty[li]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->l_empty[li]);
+        tile0 += nch;
+        const float2 s01 = fadd2(a[0], a[1]), s23 = fadd2(a[2], a[3]);
+        const float2 s4 = fadd2(s01, s23);
+        mine += s4.x + s4.y;
       }
-      tile0 += nch;
       if (!ok) break;
-      const float2 s01 = fadd2(a[0], a[1]), s23 = fadd2(a[2], a[3]);
-      const float2 s4 = fadd2(s01, s23);
-      const float mine = s4.x + s4.y;
       float *cb = comb + (xph & 1) * (kEpiWG - 1) * kRows;
       if (q < kEpiWG - 1) {
         if (!wait_or_abort(&bars->comb_empty[xph & 1], ((xph >> 1) & 1) ^ 1, bars, pc, err, 27)) break;
@@ -942,7 +985,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->comb_empty[xph & 1]);
         const int key = sp.t0 + w.kp * kBlock + klane;
-        if (key < sp.t0 + sp.len) gsum[static_cast<int64_t>(w.g) * plan.total_tokens + key] = tot;
+        const bool in = key < sp.t0 + sp.len;
+        const float rows = static_cast<float>(plan.hq * sp.n_q);
+        if (plan.direct) {
+          if (in) scores[key] = is_mm(modality[key]) ? tot / rows : 0.f;
+        } else {
+          if (in) gsum[static_cast<int64_t>(w.g) * plan.total_tokens + key] = tot;
+          if (plan.counted) {
+            __threadfence();
+            __syncwarp();
+            const int shift = 4 * (static_cast<int>(pc.rank) * 4 + quad);   // this warp's 32 keys of the block
+            uint32_t before = 0;
+            if (lane == 0) before = atomicAdd(counters + sp.blk0 + w.kp, 1u << shift);
+            before = (__shfl_sync(0xffffffffu, before, 0) >> shift) & 15u;
+            if (before == static_cast<uint32_t>(plan.hkv - 1)) {
+              __threadfence();
+              if (in) {
+                float acc = 0.f;
+                for (int g = 0; g < plan.hkv; ++g) acc += __ldcg(gsum + static_cast<int64_t>(g) * plan.total_tokens + key);
+                scores[key] = is_mm(modality[key]) ? acc / rows : 0.f;
+              }
+            }
+          }
+        }
       }
       ++xph;
     }
@@ -1062,6 +1127,7 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
   uint8_t *qp = wsb + L.qp_off;
   float *gsum = reinterpret_cast<float *>(wsb + L.gsum_off);
   uint32_t *mask_words = reinterpret_cast<uint32_t *>(wsb + L.mask_off);
+  uint32_t *counters = reinterpret_cast<uint32_t *>(wsb + kCounterOff);
 
   if (once_per_device(g_attr_done, [] {
         cudaError_t e = cudaFuncSetAttribute(score_rowstats_kernel<false>,
@@ -1098,7 +1164,9 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
     P.scale2 = kScale2Tc;
     P.causal = seqs->softmax_domain == APACK_SOFTMAX_CAUSAL_ROW;
     int64_t qrows = 0, flat = 0, nb_max = 0;
-    int units2 = 0, blocks = 0;
+    int64_t chunks2 = 0;       // pass 2: (key block, query chunk) products of one head group
+    int blocks = 0;
+    bool unscored = false;     // a sequence without query rows: its scores are zeros that no unit writes
     for (int i = 0; i < ns; ++i) {
       const int b = s0 + i;
       SeqPlan &sp = P.seq[i];
@@ -1116,8 +1184,8 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
       blocks += sp.nb;
       flat += pass1_items(sp, hkv);
       if (sp.nb > nb_max) nb_max = sp.nb;
-      sp.unit_begin = units2;
-      if (sp.rows_pad > 0) units2 += ((sp.len + kBlock - 1) / kBlock) * hkv;
+      if (sp.rows_pad > 0) chunks2 += static_cast<int64_t>((sp.len + kBlock - 1) / kBlock) * (sp.rows_pad / kChunk);
+      if (sp.rows_pad == 0 && sp.len > 0) unscored = true;
     }
     // Pass 1: equal ranges of the flat (row group, key block) items per pair; a range must stay at
     // least ceil(nb_max / (kPairSlots - 1)) items long so that a row group meets at most kPairSlots
@@ -1131,56 +1199,66 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
       if (pairs1 < 1) pairs1 = 1;
     }
     P.pairs = static_cast<int32_t>(pairs1);
-    // repack the query rows of this launch's sequences and write pass 1's key masks
+    // Pass 2: units of one head group, or of every group, which saves the group sums' round trip and the
+    // hand-over between the warpgroups once per group (about a chunk's time), as long as the longer units
+    // do not leave pairs idle in the last round.  10 minutes, 256 query rows (529 blocks, 7 chunks):
+    // 28 (7 + 1) = 224 chunk times against 7 (28 + 1) = 203; 2 minutes, 128 rows: 30 against 34.
+    const int64_t chunks_avg = blocks > 0 ? (chunks2 + blocks - 1) / blocks : 0;
+    const int64_t rounds1 = (static_cast<int64_t>(blocks) * hkv + max_pairs - 1) / max_pairs;
+    const int64_t rounds_all = (blocks + max_pairs - 1) / max_pairs;
+    const bool all_groups = hkv > 1 && !unscored && rounds_all * (hkv * chunks_avg + 1) <= rounds1 * (chunks_avg + 1);
+    P.unit_groups = all_groups ? hkv : 1;
+    P.direct = all_groups || (hkv == 1 && !unscored);
+    // The count and the re-read take about 2 us of a warpgroup, which is what the final kernel takes:
+    // hidden neither way, but a launch saved, when every pair has one unit; with more units per pair it
+    // would hold each of them up (two-minute schedule: 499 us with the kernel, 515 us counted).
+    P.counted = !P.direct && !unscored && static_cast<int64_t>(blocks) * hkv <= max_pairs && blocks <= kMaxCounted &&
+                hkv <= kMaxCountedGroups;
+    const bool final_kernel = !P.direct && !P.counted;
+    int units2 = 0;
+    for (int i = 0; i < ns; ++i) {
+      SeqPlan &sp = P.seq[i];
+      sp.unit_begin = units2;
+      if (sp.rows_pad > 0) units2 += sp.nb * (all_groups ? 1 : hkv);
+    }
+    // repack the query rows of this launch's sequences, write pass 1's key masks and zero the counters
     const int64_t n_words = static_cast<int64_t>(blocks) * (kBlock / 32);
     if (qrows > 0) {
       const int64_t n_vec = qrows * 16;
       if (check_cuda(launch_pdl(q_pack_kernel, dim3(static_cast<unsigned>((n_vec + n_words + 255) / 256)), dim3(256), 0,
                                 stream, P, static_cast<const uint4 *>(q), reinterpret_cast<uint4 *>(qp), qp_base, n_vec,
-                                seqs->modality, mask_words, n_words)) != APACK_OK)
+                                seqs->modality, mask_words, n_words, counters)) != APACK_OK)
         return APACK_ECUDA;
       count_launches(1);
     }
     if (flat > 0) {
-      const unsigned grid = static_cast<unsigned>(2 * pairs1);
-      const uint32_t *mw = mask_words;
-      const cudaError_t e = P.causal ? launch_pdl(score_rowstats_kernel<true>, dim3(grid), dim3(kThreads), kSmemBytes,
-                                                  stream, qmap, kmap, P, mw, part, err)
-                                     : launch_pdl(score_rowstats_kernel<false>, dim3(grid), dim3(kThreads), kSmemBytes,
-                                                  stream, qmap, kmap, P, mw, part, err);
+      const cudaError_t e = launch_pdl(P.causal ? score_rowstats_kernel<true> : score_rowstats_kernel<false>,
+                                       dim3(static_cast<unsigned>(2 * pairs1)), dim3(kThreads), kSmemBytes, stream, qmap,
+                                       kmap, P, mask_words, part, err);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
     if (qrows > 0) {
-      const unsigned blocks = static_cast<unsigned>((qrows * 32 + 255) / 256);   // one warp per packed row
-      const uint16_t *qp16 = reinterpret_cast<const uint16_t *>(qp);
-      const uint8_t *k8 = static_cast<const uint8_t *>(k);
-      const float2 *pc = part;
-      const int64_t qb = qp_base;
-      const cudaError_t e =
-          P.causal ? launch_pdl(lse_merge_kernel<true>, dim3(blocks), dim3(256), 0, stream, P, pc, qp16, k8,
-                                k_token_stride, static_cast<const uint8_t *>(seqs->modality), nlse2, qb, qrows)
-                   : launch_pdl(lse_merge_kernel<false>, dim3(blocks), dim3(256), 0, stream, P, pc, qp16, k8,
-                                k_token_stride, static_cast<const uint8_t *>(seqs->modality), nlse2, qb, qrows);
+      const cudaError_t e = launch_pdl(P.causal ? lse_merge_kernel<true> : lse_merge_kernel<false>,
+                                       dim3(static_cast<unsigned>(qrows / kMergeThreads)), dim3(kMergeThreads), 0, stream,
+                                       P, part, reinterpret_cast<const uint16_t *>(qp), static_cast<const uint8_t *>(k),
+                                       k_token_stride, seqs->modality, nlse2, qp_base);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
-    // Pass 2 units: (256 keys, head group), dealt round-robin to the pairs.
+    // Pass 2 units are dealt round-robin to the pairs.
     P.total_units = units2;
     if (units2 > 0) {
       const int pairs2 = units2 < max_pairs ? units2 : max_pairs;
-      const unsigned grid = static_cast<unsigned>(2 * pairs2);
-      const float *nl = nlse2;
-      const cudaError_t e = P.causal ? launch_pdl(score_colsum_kernel<true>, dim3(grid), dim3(kThreads), kSmemBytes,
-                                                  stream, qmap, kmap, P, nl, gsum, err)
-                                     : launch_pdl(score_colsum_kernel<false>, dim3(grid), dim3(kThreads), kSmemBytes,
-                                                  stream, qmap, kmap, P, nl, gsum, err);
+      const cudaError_t e = launch_pdl(P.causal ? score_colsum_kernel<true> : score_colsum_kernel<false>,
+                                       dim3(static_cast<unsigned>(2 * pairs2)), dim3(kThreads), kSmemBytes, stream, qmap,
+                                       kmap, P, nlse2, gsum, counters, seqs->modality, scores, err);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
     const int64_t t_begin = P.seq[0].t0;
     const int64_t n_tok = static_cast<int64_t>(P.seq[ns - 1].t0) + P.seq[ns - 1].len - t_begin;
-    if (n_tok > 0) {
+    if (n_tok > 0 && final_kernel) {
       const float *gs = gsum;
       if (check_cuda(launch_pdl(score_finalize_kernel, dim3(static_cast<unsigned>((n_tok + 255) / 256)), dim3(256), 0,
                                 stream, P, static_cast<const uint8_t *>(seqs->modality), gs, scores, t_begin,

@@ -154,6 +154,27 @@ def test_scores_match_oracle(ap, lens, nqs, hq, hkv):
         assert tot == pytest.approx(1.0 if S and nqs[s] else 0.0, abs=1e-4)
 
 
+@pytest.mark.parametrize("domain", [0, 1])
+@pytest.mark.parametrize("lens,nqs,hq,hkv", [
+    ([19000], [20], 28, 4),                 # units of every head group: the unit writes the scores
+    ([19000, 257], [20, 0], 28, 4),         # a sequence without query rows: the final kernel
+    ([9000], [20], 28, 4),                  # more units than CTA pairs: the final kernel
+    ([4000, 0, 255], [40, 0, 40], 28, 4),   # one unit per pair: the last of a key block adds the groups
+    ([1000], [40], 16, 16),                 # as many, but more groups than the counters count
+    ([5000], [40], 8, 1),                   # one head group
+])
+def test_column_pass_modes(ap, lens, nqs, hq, hkv, domain):
+    """The ways in which the head groups' sums meet, equal to the oracle (tolerance of
+    test_narrow_path_head_layouts_and_row_counts) and the same bits in every call."""
+    rng = np.random.default_rng(sum(lens) + hq + domain)
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
+    check_scores(got, ref, strict_rel=2e-4)
+    again = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    assert got.tobytes() == again.tobytes()
+
+
 # ------------------------------------------------------------------------------ causal-row domain
 
 CAUSAL_SHAPES = [
