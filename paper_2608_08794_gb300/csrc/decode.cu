@@ -41,8 +41,12 @@ constexpr int kStageBytes = 32768;                // K (and V) bytes per stage: 
 constexpr int kDecRows = 8;                       // query rows per KV head group (G <= 8)
 constexpr size_t kDecSmem = static_cast<size_t>(kDecStages) * 2 * kStageBytes + 2 * kDecStages * sizeof(uint64_t) +
                             (kDecConsumers * 8 * kDecRows + kDecConsumers * kDecRows) * sizeof(float) + 16;
-constexpr int kDecCombineThreads = 512;
-constexpr int kDecCombineWarps = kDecCombineThreads / 32;
+// Warps of a combine CTA: 4 when every sequence of the launch has at most 40 chunks (one round of loads
+// per warp), else 16.  16 caches of 600 to 12,000 tokens (9 chunks on average): 31.5 us a call with 16
+// warps, most of them idle and all of them in the last merge, 27.7 us with 4 (and a first
+// unit of its own per chunk CTA, which gives 0.2 us of that).
+constexpr int kDecCombineFew = 4, kDecCombineMany = 16;
+constexpr int kDecCombineBatch = 10;              // chunk partials loaded before they are merged
 
 __device__ __forceinline__ void bf16x4_to_f32(const uint2 &w, float (&f)[4]) {
   f[0] = __uint_as_float(w.x << 16);
@@ -282,30 +286,30 @@ __global__ void __launch_bounds__(kDecThreads, 1)
   }
 }
 
-// One CTA per (sequence, query head): merge the sequence's chunks.  Warp w folds chunks
-// w, w + 16, w + 32, ... in that order (lane: features [4 lane, 4 lane + 4)); the warps
+// One CTA of WARPS warps per (sequence, query head): merge the sequence's chunks.  Warp w folds chunks
+// w, w + WARPS, w + 2 WARPS, ... in that order (lane: features [4 lane, 4 lane + 4)); the warps
 // then merge in warp order.  A sequence with no cached token gets zeros.  The CTA of query
 // head 0 also zeroes the sequence's stage-claim counter for the next call (the chunk kernel,
 // the counter's only user, is complete here).
-__global__ void __launch_bounds__(kDecCombineThreads)
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
     decode_combine_kernel(const __grid_constant__ DecPlan plan, const float *__restrict__ opart,
                           const float2 *__restrict__ mlpart, float *__restrict__ out, unsigned int *claims) {
-  __shared__ __align__(16) float wo[kDecCombineWarps][128];
-  __shared__ float2 wml[kDecCombineWarps];
+  __shared__ __align__(16) float wo[WARPS][128];
+  __shared__ float2 wml[WARPS];
   pdl_wait_and_release();                   // the chunk kernel's partials are complete and visible
   const int s = blockIdx.x / plan.hq, hh = blockIdx.x % plan.hq;
   if (hh == 0 && threadIdx.x == 0) claims[s] = 0u;
   const DecSeq &sq = plan.seq[s];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
-  constexpr int kBatch = 10;                // chunk partials loaded before they are merged (one
-                                            // round for up to 160 chunks)
-  for (int c0 = warp; c0 < sq.nchunks; c0 += kDecCombineWarps * kBatch) {
+  constexpr int kBatch = kDecCombineBatch;
+  for (int c0 = warp; c0 < sq.nchunks; c0 += WARPS * kBatch) {
     float2 ml[kBatch];
     float4 a[kBatch];
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
-      const int cc = c0 + i * kDecCombineWarps;
+      const int cc = c0 + i * WARPS;
       const int64_t idx = static_cast<int64_t>(sq.chunk_begin + cc) * plan.hq + hh;
       ml[i] = cc < sq.nchunks ? mlpart[idx] : make_float2(-INFINITY, 0.f);
       a[i] = cc < sq.nchunks ? *reinterpret_cast<const float4 *>(opart + idx * 128 + lane * 4)
@@ -322,7 +326,7 @@ __global__ void __launch_bounds__(kDecCombineThreads)
   __syncthreads();
   if (warp == 0) {
     float M = -INFINITY, L = 0.f, O[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int w = 0; w < kDecCombineWarps; ++w) {
+    for (int w = 0; w < WARPS; ++w) {
       const float4 a = *reinterpret_cast<const float4 *>(&wo[w][lane * 4]);
       const float o2[4] = {a.x, a.y, a.z, a.w};
       merge_state(M, L, O, wml[w].x, wml[w].y, o2);
@@ -434,7 +438,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     P.group = num_q_heads / num_kv_heads;
     P.chunk = chunk;                    // whole 128-key tiles
     P.scale2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(APACK_HEAD_DIM)));
-    int chunks = 0;
+    int chunks = 0, max_chunks = 0;
     for (int i = 0; i < ns; ++i) {
       DecSeq &d = P.seq[i];
       d.t0 = cu_seqlens_h[s0 + i];
@@ -442,6 +446,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
       d.chunk_begin = chunks;
       d.nchunks = (d.len + chunk - 1) / chunk;
       chunks += d.nchunks;
+      max_chunks = std::max(max_chunks, d.nchunks);
     }
     P.total_chunks = chunks;
     float *op = opart + chunk_base * num_q_heads * 128;
@@ -461,8 +466,9 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     }
     // programmatic dependent launch: the combine's CTAs are scheduled while the chunk kernel
     // drains and wait (griddepcontrol.wait) for its completion before reading the partials
-    if (check_cuda(launch_pdl(decode_combine_kernel, dim3(ns * num_q_heads), dim3(kDecCombineThreads), 0, s, P,
-                              static_cast<const float *>(op), static_cast<const float2 *>(mp),
+    const bool few = max_chunks <= kDecCombineFew * kDecCombineBatch;
+    if (check_cuda(launch_pdl(few ? decode_combine_kernel<kDecCombineFew> : decode_combine_kernel<kDecCombineMany>,
+                              dim3(ns * num_q_heads), dim3(32 * (few ? kDecCombineFew : kDecCombineMany)), 0, s, P, op, mp,
                               out + static_cast<int64_t>(s0) * num_q_heads * 128, claims + s0)) != APACK_OK)
       return APACK_ECUDA;
     count_launches(1);

@@ -5,8 +5,9 @@
 //
 // About one CTA per SM (each sequence gets CTAs in proportion to its length), all KV heads.  A
 // stage is one KV head of one 128-key tile; the CTAs of a sequence claim its stages in order
-// from a counter in the workspace (tile-major, heads within a tile), so that CTAs on SMs that
-// stream faster take more of them and all finish together.  Each CTA folds every stage it
+// from a counter in the workspace (tile-major, heads within a tile; each CTA's first two are its own,
+// without the counter's round trip), so that CTAs on SMs that stream faster take more of them and all
+// finish together.  Each CTA folds every stage it
 // claims into its running per-head state, so it still writes one partial per query head;
 // which CTA takes which stage varies from call to call, and with it the last bits of the
 // result.  The combine kernel resets the counter for the next call.  A stage's K rows and V
@@ -207,11 +208,13 @@ __global__ void __launch_bounds__(kDThreads, 1)
     if (lane == 0) {
       tma_prefetch_desc(&kmap);
       tma_prefetch_desc(&vmap);
-      // claims run two stages ahead of the loads (an atomic's round trip is about a stage's
-      // time); one thread's claims on one counter return increasing units
+      // a CTA's first two units are its own (c and n + c of the sequence's n CTAs), the rest are claimed;
+      // claims run two stages ahead of the loads (an atomic's round trip is about a stage's time); one
+      // thread's claims on one counter return increasing units
       unsigned int *claim = claims + s;
-      int next = static_cast<int>(atomicAdd(claim, 1u));   // stage 0's unit
-      int next2 = static_cast<int>(atomicAdd(claim, 1u));  // stage 1's
+      const int rank = c - sq.chunk_begin, own = 2 * sq.nchunks;
+      int next = rank;                                      // stage 0's unit
+      int next2 = sq.nchunks + rank;                        // stage 1's
       int unit[2] = {0, 0};                       // units of the last two claimed stages (by n & 1)
       int n_end = -1;                             // the number of claimed stages, once known
       int last = -1;                              // the last item issued with a load
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
             continue;                              // no load: V(n - 1) is the last item
           }
           next = next2;
-          next2 = static_cast<int>(atomicAdd(claim, 1u));  // stage n + 2's unit
+          next2 = own + static_cast<int>(atomicAdd(claim, 1u));   // stage n + 2's unit
           unit[n & 1] = u;
           bars->info[r] = u;
           mbar_arrive(&bars->info_full[r]);

@@ -83,6 +83,20 @@ def test_decode_attention_matches_oracle(ap, lens, hq, hkv):
         assert got.tobytes() == again.tobytes()
 
 
+@pytest.mark.parametrize("hq,hkv", [(28, 4), (8, 1)])
+@pytest.mark.parametrize("lens", [
+    [128 * 152],                    # one tile per chunk: as many chunks as the wide combine merges in one round
+    [128 * 40], [128 * 41 - 1],     # 40 chunks, the most of the narrow combine's rounds, and 41
+    [1, 127, 129, 2, 128 * 3],      # CTAs whose second own unit lies past the sequence
+])
+def test_decode_attention_chunk_counts(ap, lens, hq, hkv):
+    rng = np.random.default_rng(sum(lens) + hq)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    T = int(cu[-1])
+    q, k, v = bits(rng, (len(lens), hq, 128), 1.5), bits(rng, (T, hkv, 128)), bits(rng, (T, hkv, 128))
+    check(run(ap, cu, q, k, v, hq, hkv), oracle.decode_attention(q, k, v, cu, hq, hkv))
+
+
 def test_decode_attention_strided_rows_and_uniform_keys(ap):
     rng = np.random.default_rng(7)
     cu = np.array([0, 777, 1500], np.int32)
