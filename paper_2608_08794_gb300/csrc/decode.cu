@@ -55,6 +55,24 @@ __device__ __forceinline__ void bf16x4_to_f32(const uint2 &w, float (&f)[4]) {
   f[3] = __uint_as_float(w.y & 0xFFFF0000u);
 }
 
+// R consecutive floats of shared memory.
+template <int R>
+__device__ __forceinline__ void load_row(const float *p, float (&v)[R]) {
+  if (R >= 4) {
+#pragma unroll
+    for (int j = 0; j + 3 < R; j += 4) {
+      const float4 x = *reinterpret_cast<const float4 *>(p + j);
+      v[j] = x.x;
+      v[j + 1] = x.y;
+      v[j + 2] = x.z;
+      v[j + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[j] = p[j];
+  }
+}
+
 // Merge (m2, l2, o2) into (m1, l1, o1) (log2 units).
 __device__ __forceinline__ void merge_state(float &m1, float &l1, float (&o1)[4], float m2, float l2,
                                             const float (&o2)[4]) {
@@ -97,6 +115,10 @@ __device__ __forceinline__ void decode_issue_stage(const DecSeq &sq, const uint8
   }
 }
 
+// R: query rows per KV head group that the kernel works on, 1, 2, 4 or 8 (G rounded up): with 8 for
+// every group, heads of one or four rows spent most of their arithmetic on rows of zeros.  135,000
+// cached tokens: 129 -> 83.5 us (8/8 heads; reading the cache takes 81.4), 130 -> 92.7 us (32/8 heads).
+template <int R>
 __global__ void __launch_bounds__(kDecThreads, 1)
     decode_chunk_kernel(const __grid_constant__ DecPlan plan, const uint16_t *__restrict__ q,
                         const uint8_t *__restrict__ k, const uint8_t *__restrict__ v, int64_t kv_stride,
@@ -129,6 +151,9 @@ __global__ void __launch_bounds__(kDecThreads, 1)
     fence_mbar_init();
   }
   __syncthreads();
+  // launched as a programmatic dependent: the set-up runs beside the previous launch; the caches, q and
+  // the partials (which the previous call's combine reads) are touched once it has completed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   volatile int *abort_v = abort_flag;
   int issued = 0;
   if (loader)
@@ -136,22 +161,23 @@ __global__ void __launch_bounds__(kDecThreads, 1)
       decode_issue_stage(sq, k, v, kv_stride, row, stage_tok, tb, te, issued, stage_base, full);
 
   const int h = warp % hkv, grp = warp / hkv;
-  const int cl = (lane >> 2) & 7;       // after the reduce-scatter this lane holds row cl
-  float qf[kDecRows][4];                // query rows, lane-permuted: slot j holds row j ^ cl
+  constexpr int kLog = R == 8 ? 3 : R == 4 ? 2 : R == 2 ? 1 : 0;
+  const int cl = lane >> (5 - kLog);    // after the reduce-scatter this lane holds row cl
+  float qf[R][4];                       // query rows, lane-permuted: slot j holds row j ^ cl
   const uint16_t *qg = q + (static_cast<int64_t>(s) * plan.hq + h * G) * 128 + lane * 4;
 #pragma unroll
-  for (int j = 0; j < kDecRows; ++j) {
+  for (int j = 0; j < R; ++j) {
     const int r = j ^ cl;
     uint2 w = make_uint2(0, 0);
     if (r < G) w = __ldg(reinterpret_cast<const uint2 *>(qg + r * 128));
     bf16x4_to_f32(w, qf[j]);
   }
-  float o[kDecRows][4];
+  float o[R][4];
 #pragma unroll
-  for (int j = 0; j < kDecRows; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+  for (int j = 0; j < R; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
   float m_own = -INFINITY, l_own = 0.f;
-  float *wps = ps + warp * 8 * kDecRows;
-  float *wsc = sc + warp * kDecRows;
+  float *wps = ps + warp * 8 * R;
+  float *wsc = sc + warp * R;
   for (int n = 0; n < nst; ++n) {
     const int slot = n % kDecStages;
     // the decision to go on is warp-uniform: every lane waited, and all must have succeeded
@@ -173,23 +199,30 @@ __global__ void __launch_bounds__(kDecThreads, 1)
       for (int i = 0; i < 8; ++i) {
         float kf[4];
         bf16x4_to_f32(i < valid ? *reinterpret_cast<const uint2 *>(ks + i * row) : make_uint2(0, 0), kf);
-        float acc[kDecRows];
-#pragma unroll
-        for (int j = 0; j < kDecRows; j += 2) {
+        float acc[R];
+        if (R == 1) {
           float2 a = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) a = ffma2(make_float2(kf[e], kf[e]), make_float2(qf[j][e], qf[j + 1][e]), a);
-          acc[j] = a.x;
-          acc[j + 1] = a.y;
+          for (int e = 0; e < 4; e += 2) a = ffma2(make_float2(kf[e], kf[e + 1]), make_float2(qf[0][e], qf[0][e + 1]), a);
+          acc[0] = a.x + a.y;
+        } else {
+#pragma unroll
+          for (int j = 0; j + 1 < R; j += 2) {
+            float2 a = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a = ffma2(make_float2(kf[e], kf[e]), make_float2(qf[j][e], qf[j + 1][e]), a);
+            acc[j] = a.x;
+            acc[j + 1] = a.y;
+          }
         }
         // slot e and the partner's slot e + half hold the same row at every level
+        int mask = 16;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e + 4], 16);
+        for (int half = R / 2; half >= 1; half /= 2, mask /= 2)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e + 2], 8);
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[1], 4);
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+          for (int e = 0; e < half; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e + half], mask);
+#pragma unroll
+        for (; mask >= 1; mask /= 2) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], mask);
         x[i] = i < valid ? acc[0] * plan.scale2 : -INFINITY;
       }
       // online softmax of row cl over these keys (key 0 of the group is valid)
@@ -203,37 +236,42 @@ __global__ void __launch_bounds__(kDecThreads, 1)
       for (int i = 0; i < 8; ++i) {
         const float p = ex2_approx(x[i] - mn);
         psum += p;
-        wps[i * kDecRows + cl] = p;        // the four lanes of a row write the same value
+        wps[i * R + cl] = p;               // the lanes of a row write the same value
       }
       wsc[cl] = scale;
       l_own = l_own * scale + psum;
       m_own = mn;
       __syncwarp();
-      {
-        const float4 sa = *reinterpret_cast<const float4 *>(wsc);
-        const float4 sb = *reinterpret_cast<const float4 *>(wsc + 4);
-        const float sr[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
 #pragma unroll
-        for (int j = 0; j < kDecRows; ++j)
+      for (int j = 0; j < R; ++j) {
+        const float f = wsc[j];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) o[j][e] *= sr[j];
+        for (int e = 0; e < 4; ++e) o[j][e] *= f;
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         float vf[4];
         bf16x4_to_f32(i < valid ? *reinterpret_cast<const uint2 *>(vs + i * row) : make_uint2(0, 0), vf);
-        const float4 pa = *reinterpret_cast<const float4 *>(wps + i * kDecRows);
-        const float4 pb = *reinterpret_cast<const float4 *>(wps + i * kDecRows + 4);
-        const float pr[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+        float pr[R];
+        load_row<R>(wps + i * R, pr);
+        if (R == 1) {
 #pragma unroll
-        for (int j = 0; j < kDecRows; j += 2)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 r2 = ffma2(make_float2(pr[j], pr[j + 1]), make_float2(vf[e], vf[e]),
-                                    make_float2(o[j][e], o[j + 1][e]));
-            o[j][e] = r2.x;
-            o[j + 1][e] = r2.y;
+          for (int e = 0; e < 4; e += 2) {
+            const float2 r2 = ffma2(make_float2(pr[0], pr[0]), make_float2(vf[e], vf[e + 1]), make_float2(o[0][e], o[0][e + 1]));
+            o[0][e] = r2.x;
+            o[0][e + 1] = r2.y;
           }
+        } else {
+#pragma unroll
+          for (int j = 0; j + 1 < R; j += 2)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 r2 = ffma2(make_float2(pr[j], pr[j + 1]), make_float2(vf[e], vf[e]),
+                                      make_float2(o[j][e], o[j + 1][e]));
+              o[j][e] = r2.x;
+              o[j + 1][e] = r2.y;
+            }
+        }
       }
     }
     __syncwarp();                        // this warp is done with the stage and its scratch
@@ -258,32 +296,45 @@ __global__ void __launch_bounds__(kDecThreads, 1)
       mbar_wait(&full[n % kDecStages], (n / kDecStages) & 1u, kWaitLimitNs / 4);
   __syncthreads();
   if (*abort_v) return;
-  // merge the warps of each head in group order; the stages are free now
+  // merge the warps of each head in group order, one (head, row) per warp and round; the stages are
+  // free now
   float *wo = reinterpret_cast<float *>(stage_base);                   // [warp][row][128]
-  float2 *wml = reinterpret_cast<float2 *>(wo + kDecConsumers * kDecRows * 128);
+  float2 *wml = reinterpret_cast<float2 *>(wo + kDecConsumers * R * 128);
 #pragma unroll
-  for (int j = 0; j < kDecRows; ++j)
-    *reinterpret_cast<float4 *>(wo + (warp * kDecRows + j) * 128 + lane * 4) =
+  for (int j = 0; j < R; ++j)
+    *reinterpret_cast<float4 *>(wo + (warp * R + j) * 128 + lane * 4) =
         make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
-  if ((lane & 3) == 0) wml[warp * kDecRows + cl] = make_float2(m_own, l_own);
+  if ((lane & (32 / R - 1)) == 0) wml[warp * R + cl] = make_float2(m_own, l_own);
   __syncthreads();
-  if (grp == 0) {
-    for (int j = 0; j < G; ++j) {
-      float m1 = wml[warp * kDecRows + j].x, l1 = wml[warp * kDecRows + j].y;
-      const float4 a = *reinterpret_cast<const float4 *>(wo + (warp * kDecRows + j) * 128 + lane * 4);
-      float o1[4] = {a.x, a.y, a.z, a.w};
-      for (int g2 = 1; g2 < kDecConsumers / hkv; ++g2) {
-        const int w2 = g2 * hkv + h;
-        const float2 ml2 = wml[w2 * kDecRows + j];
-        const float4 b = *reinterpret_cast<const float4 *>(wo + (w2 * kDecRows + j) * 128 + lane * 4);
-        const float o2[4] = {b.x, b.y, b.z, b.w};
-        merge_state(m1, l1, o1, ml2.x, ml2.y, o2);
-      }
-      const int64_t hq_idx = static_cast<int64_t>(c) * plan.hq + h * G + j;
-      *reinterpret_cast<float4 *>(opart + hq_idx * 128 + lane * 4) = make_float4(o1[0], o1[1], o1[2], o1[3]);
-      if (lane == 0) mlpart[hq_idx] = make_float2(m1, l1);
+  for (int e = warp; e < hkv * G; e += kDecConsumers) {
+    const int hh = e / G, j = e - hh * G;
+    float m1 = wml[hh * R + j].x, l1 = wml[hh * R + j].y;
+    const float4 a = *reinterpret_cast<const float4 *>(wo + (hh * R + j) * 128 + lane * 4);
+    float o1[4] = {a.x, a.y, a.z, a.w};
+    for (int g2 = 1; g2 < kDecConsumers / hkv; ++g2) {
+      const int w2 = g2 * hkv + hh;
+      const float2 ml2 = wml[w2 * R + j];
+      const float4 b = *reinterpret_cast<const float4 *>(wo + (w2 * R + j) * 128 + lane * 4);
+      const float o2[4] = {b.x, b.y, b.z, b.w};
+      merge_state(m1, l1, o1, ml2.x, ml2.y, o2);
     }
+    const int64_t hq_idx = static_cast<int64_t>(c) * plan.hq + e;
+    *reinterpret_cast<float4 *>(opart + hq_idx * 128 + lane * 4) = make_float4(o1[0], o1[1], o1[2], o1[3]);
+    if (lane == 0) mlpart[hq_idx] = make_float2(m1, l1);
   }
+}
+
+template <int R>
+cudaError_t launch_chunk(int grid, cudaStream_t stream, const DecPlan &P, const uint16_t *q, const uint8_t *k,
+                         const uint8_t *v, int64_t kv_stride, float *opart, float2 *mlpart, DeviceError *err) {
+  static std::atomic<uint64_t> attr{0};
+  const cudaError_t e = once_per_device(attr, [] {
+    return cudaFuncSetAttribute(decode_chunk_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kDecSmem));
+  });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(decode_chunk_kernel<R>, dim3(grid), dim3(kDecThreads), kDecSmem, stream, P, q, k, v, kv_stride,
+                    opart, mlpart, err);
 }
 
 // One CTA of WARPS warps per (sequence, query head): merge the sequence's chunks.  Warp w folds chunks
@@ -340,14 +391,29 @@ __global__ void __launch_bounds__(32 * WARPS)
 // The tensor-core chunk kernel takes Hkv = 2 or 4 with at most 8 query heads per KV head.
 bool decode_tc_applies(int32_t hq, int32_t hkv) { return (hkv == 2 || hkv == 4) && hq / hkv <= kDecRows; }
 
-// Keys per chunk: about one CTA per SM over the whole batch, whole 128-key tiles (a multiple of
-// every stage size of both chunk kernels).
-int decode_chunk_keys(int64_t total_tokens, int32_t hkv) {
-  (void)hkv;
-  const int64_t ctas = device_sm_count();
-  int64_t c = (total_tokens + ctas - 1) / std::max<int64_t>(1, ctas);
-  c = (c + 127) / 128 * 128;
-  return static_cast<int>(std::min<int64_t>(std::max<int64_t>(c, 128), 1 << 20));
+// Keys per chunk, whole 128-key tiles (a multiple of every stage size of both chunk kernels): about one
+// CTA per SM over the whole batch, and then as many as bring every launch (kSeqsPerLaunch sequences) down
+// to one CTA per SM, within 1/16: a last chunk per sequence that starts a second round of CTAs costs as
+// much as the first (48 caches of 100 to 3,000 tokens, 28/4 heads: 55.2 -> 38.6 us).
+int decode_chunk_keys(int32_t num_seqs, const int32_t *cu_seqlens_h) {
+  const int64_t ctas = std::max(1, device_sm_count());
+  const int64_t total = num_seqs > 0 ? cu_seqlens_h[num_seqs] : 0;
+  auto whole = [](int64_t c) { return std::max<int64_t>(128, (c + 127) / 128 * 128); };
+  int64_t c = whole((total + ctas - 1) / ctas);
+  for (int s0 = 0; s0 < num_seqs; s0 += kSeqsPerLaunch) {
+    const int s1 = std::min(num_seqs, s0 + kSeqsPerLaunch);
+    for (;;) {
+      int64_t n = 0, longest = 0;
+      for (int b = s0; b < s1; ++b) {
+        const int64_t len = cu_seqlens_h[b + 1] - cu_seqlens_h[b];
+        n += (len + c - 1) / c;
+        longest = std::max(longest, len);
+      }
+      if (n <= ctas || c >= longest) break;
+      c = whole(c + std::max<int64_t>(1, c / 16));
+    }
+  }
+  return static_cast<int>(std::min<int64_t>(c, 1 << 20));
 }
 
 apack_status decode_validate(int32_t num_seqs, const int32_t *cu_seqlens_h, int32_t hq, int32_t hkv,
@@ -378,7 +444,7 @@ apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seq
   int64_t total = 0;
   const apack_status st = decode_validate(num_seqs, cu_seqlens_h, num_q_heads, num_kv_heads, &total);
   if (st != APACK_OK) return st;
-  const int chunk = decode_chunk_keys(total, num_kv_heads);
+  const int chunk = decode_chunk_keys(num_seqs, cu_seqlens_h);
   int64_t chunks = 0;
   for (int b = 0; b < num_seqs; ++b) chunks += (cu_seqlens_h[b + 1] - cu_seqlens_h[b] + chunk - 1) / chunk;
   // device error word, chunk partials o [chunks][Hq][128] and (max, sum) [chunks][Hq], one
@@ -406,7 +472,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
   size_t need = 0;
   apack_decode_workspace_size(num_seqs, cu_seqlens_h, num_q_heads, num_kv_heads, &need);
   if (ws_bytes < need) return APACK_EWORKSPACE;
-  const int chunk = decode_chunk_keys(total, num_kv_heads);
+  const int chunk = decode_chunk_keys(num_seqs, cu_seqlens_h);
   int64_t chunks_all = 0;
   for (int b = 0; b < num_seqs; ++b) chunks_all += (cu_seqlens_h[b + 1] - cu_seqlens_h[b] + chunk - 1) / chunk;
   DeviceError *err = static_cast<DeviceError *>(ws);
@@ -415,12 +481,6 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
                                               up256(static_cast<size_t>(chunks_all) * num_q_heads * 128 * sizeof(float)));
   unsigned int *claims = reinterpret_cast<unsigned int *>(
       reinterpret_cast<uint8_t *>(mlpart) + up256(static_cast<size_t>(chunks_all) * num_q_heads * sizeof(float2)));
-  static std::atomic<uint64_t> attr_done{0};
-  if (once_per_device(attr_done, [] {
-        return cudaFuncSetAttribute(decode_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(kDecSmem));
-      }) != cudaSuccess)
-    return APACK_ECUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t *q16 = static_cast<const uint16_t *>(q);
   const bool tc = decode_tc_applies(num_q_heads, num_kv_heads) && total > 0;
@@ -457,10 +517,11 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
         if (check_cuda(launch_decode_tc(chunks, s, kmap, vmap, P, qs, op, mp, claims + s0, err)) != APACK_OK)
           return APACK_ECUDA;
       } else {
-        decode_chunk_kernel<<<chunks, kDecThreads, kDecSmem, s>>>(P, qs, static_cast<const uint8_t *>(k),
-                                                                  static_cast<const uint8_t *>(v), kv_token_stride,
-                                                                  op, mp, err);
-        if (check_cuda(cudaGetLastError()) != APACK_OK) return APACK_ECUDA;
+        auto *launch = P.group > 4 ? launch_chunk<8> : P.group > 2 ? launch_chunk<4> : P.group > 1 ? launch_chunk<2>
+                                                                                                   : launch_chunk<1>;
+        if (check_cuda(launch(chunks, s, P, qs, static_cast<const uint8_t *>(k), static_cast<const uint8_t *>(v),
+                              kv_token_stride, op, mp, err)) != APACK_OK)
+          return APACK_ECUDA;
       }
       count_launches(1);
     }
