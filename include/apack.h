@@ -325,8 +325,8 @@ apack_status apack_graph_destroy(apack_graph graph);
    Hkv 2 or 4 and at most 8 query heads per KV head (the tensor-core path) the
    CTAs of a sequence claim its 128-key tiles from a counter as they go, so
    the grouping of keys into partial sums, and with it the last bits of out,
-   can differ from call to call; the other head layouts merge in a fixed
-   order.  ws: 256-byte aligned, apack_decode_workspace_size bytes (the size
+   can differ from call to call (not where the caches are so short that each
+   CTA has its own tiles); the other head layouts merge in a fixed order.  ws: 256-byte aligned, apack_decode_workspace_size bytes (the size
    depends on the device's SM count: query it on the device that runs the
    call), zeroed by the caller once before its first use: its first 16 bytes
    are a device error word read by apack_device_error, and it holds the

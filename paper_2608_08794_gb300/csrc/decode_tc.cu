@@ -7,7 +7,8 @@
 // stage is one KV head of one 128-key tile; the CTAs of a sequence claim its stages in order
 // from a counter in the workspace (tile-major, heads within a tile; each CTA's first two are its own,
 // without the counter's round trip), so that CTAs on SMs that stream faster take more of them and all
-// finish together.  Each CTA folds every stage it
+// finish together.  A launch of few chunks gives each chunk several CTAs with a share of the KV heads
+// and its own stages (no claims, so the result is the same in every call).  Each CTA folds every stage it
 // claims into its running per-head state, so it still writes one partial per query head;
 // which CTA takes which stage varies from call to call, and with it the last bits of the
 // result.  The combine kernel resets the counter for the next call.  A stage's K rows and V
@@ -145,7 +146,9 @@ __global__ void __launch_bounds__(kDThreads, 1)
   float *tmax = reinterpret_cast<float *>(smem + Lay::kOffT);
   float *msm = reinterpret_cast<float *>(smem + Lay::kOffM);
   DBars *bars = reinterpret_cast<DBars *>(smem + Lay::kOffBars);
-  const int c = blockIdx.x;
+  const int c = blockIdx.x >> plan.split_log;
+  const int heads = HKV >> plan.split_log;                   // this CTA's KV heads: h0 .. h0 + heads
+  const int h0 = (blockIdx.x - (c << plan.split_log)) * heads;
   const int s = find_chunk_seq(plan, c);
   const DecSeq &sq = plan.seq[s];
   const int G = plan.group;
@@ -213,8 +216,12 @@ __global__ void __launch_bounds__(kDThreads, 1)
       // thread's claims on one counter return increasing units
       unsigned int *claim = claims + s;
       const int rank = c - sq.chunk_begin, own = 2 * sq.nchunks;
-      int next = rank;                                      // stage 0's unit
-      int next2 = sq.nchunks + rank;                        // stage 1's
+      const bool claimed = plan.split_log == 0;
+      const int tile0 = rank * (plan.chunk / kDM);          // split: the chunk's tiles, this CTA's heads
+      const int mine = min(plan.chunk / kDM, units / HKV - tile0) * heads;
+      auto unit_of = [&](int n) { return n < mine ? (tile0 + n / heads) * HKV + h0 + n % heads : units; };
+      int next = claimed ? rank : unit_of(0);                   // stage 0's unit
+      int next2 = claimed ? sq.nchunks + rank : unit_of(1);     // stage 1's
       int unit[2] = {0, 0};                       // units of the last two claimed stages (by n & 1)
       int n_end = -1;                             // the number of claimed stages, once known
       int last = -1;                              // the last item issued with a load
@@ -237,7 +244,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
             continue;                              // no load: V(n - 1) is the last item
           }
           next = next2;
-          next2 = own + static_cast<int>(atomicAdd(claim, 1u));   // stage n + 2's unit
+          next2 = claimed ? own + static_cast<int>(atomicAdd(claim, 1u)) : unit_of(n + 2);   // stage n + 2's unit
           unit[n & 1] = u;
           bars->info[r] = u;
           mbar_arrive(&bars->info_full[r]);
@@ -503,7 +510,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
         tmem_ld16_wait(bars->tmem_base + lane_off + 32 + h * kDN, o);
 #pragma unroll
       for (int j = 0; j < kDRows; ++j)           // feature kt of row j: high plus low part
-        if (j < G)
+        if (j < G && static_cast<unsigned>(h - h0) < static_cast<unsigned>(heads))
           opart[(static_cast<int64_t>(c) * plan.hq + h * G + j) * 128 + kt] =
               __uint_as_float(o[j]) + __uint_as_float(o[j + 8]);
 #pragma unroll
@@ -522,7 +529,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
   __syncthreads();
   if (ok) {
     // one warp per (head, row): the 128 partial sums in a fixed order
-    for (int e = warp; e < HKV * G; e += kDThreads / 32) {
+    for (int e = h0 * G + warp; e < (h0 + heads) * G; e += kDThreads / 32) {
       const int h = e / G, j = e % G;
       const float4 l4 = *reinterpret_cast<const float4 *>(lsum + (h * kDRows + j) * kDM + lane * 4);
       float l = (l4.x + l4.y) + (l4.z + l4.w);

@@ -95,7 +95,9 @@ def test_decode_attention_chunk_counts(ap, lens, hq, hkv):
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     T = int(cu[-1])
     q, k, v = bits(rng, (len(lens), hq, 128), 1.5), bits(rng, (T, hkv, 128)), bits(rng, (T, hkv, 128))
-    check(run(ap, cu, q, k, v, hq, hkv), oracle.decode_attention(q, k, v, cu, hq, hkv))
+    ref = oracle.decode_attention(q, k, v, cu, hq, hkv)
+    check(run(ap, cu, q, k, v, hq, hkv), ref)
+    check(run(ap, cu, q, k, v, hq, hkv, pad_heads=1), ref)      # token rows wider than the heads
 
 
 def test_decode_attention_strided_rows_and_uniform_keys(ap):
