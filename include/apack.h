@@ -329,8 +329,10 @@ apack_status apack_graph_destroy(apack_graph graph);
    CTA has its own tiles); the other head layouts merge in a fixed order.  ws: 256-byte aligned, apack_decode_workspace_size bytes (the size
    depends on the device's SM count: query it on the device that runs the
    call), zeroed by the caller once before its first use: its first 16 bytes
-   are a device error word read by apack_device_error, and it holds the
-   claim counters, which every call leaves at zero.  A device-side wait that
+   are a device error word read by apack_device_error, and its end (of the
+   ws_bytes passed: pass the same for one workspace) holds the claim
+   counters, which every call leaves at zero; caches may grow and shrink
+   from call to call.  A device-side wait that
    runs out records APACK_ETIMEOUT there.  Two kernel launches per 64
    sequences; no allocation, no synchronisation. */
 apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seqlens_h, int32_t num_q_heads,

@@ -483,8 +483,10 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
   float *opart = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + 256);
   float2 *mlpart = reinterpret_cast<float2 *>(static_cast<uint8_t *>(ws) + 256 +
                                               up256(static_cast<size_t>(chunks_all) * num_q_heads * 128 * sizeof(float)));
-  unsigned int *claims = reinterpret_cast<unsigned int *>(
-      reinterpret_cast<uint8_t *>(mlpart) + up256(static_cast<size_t>(chunks_all) * num_q_heads * sizeof(float2)));
+  // the claim counters lie at the end of the workspace that the caller passed, not after this call's
+  // partials: they stay where they are, and zero, when the caches grow or shrink between calls
+  const size_t claims_off = (ws_bytes - up256(static_cast<size_t>(num_seqs) * sizeof(unsigned int))) & ~static_cast<size_t>(255);
+  unsigned int *claims = reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(ws) + claims_off);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t *q16 = static_cast<const uint16_t *>(q);
   const bool tc = decode_tc_applies(num_q_heads, num_kv_heads) && total > 0;

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
           // publish stage n's record (its unit, or the end of the claims) before its K load
           const int u = next;
           const int r = n % kDInfo;
-          if (u >= units) {
+          if (static_cast<unsigned>(u) >= static_cast<unsigned>(units)) {   // a counter left dirty ends the claims too
             bars->info[r] = -1;
             mbar_arrive(&bars->info_full[r]);
             n_end = n;

@@ -200,6 +200,28 @@ def test_decode_attention_repeated_calls_on_one_workspace(ap):
         check(out.cpu().numpy(), ref)
 
 
+def test_decode_attention_growing_and_shrinking_caches_on_one_workspace(ap):
+    # The number of chunk partials follows the cache; the claim counters must not end up on partials
+    # of an earlier call (19,456 tokens: 152 chunks of 128 keys, one more: 77 of 256).
+    rng = np.random.default_rng(31)
+    T = 40000
+    q, k, v = bits(rng, (2, 28, 128)), bits(rng, (T, 4, 128), 1.5), bits(rng, (T, 4, 128))
+    kd = torch.from_numpy(k.reshape(T, -1).view(np.int16)).cuda()
+    vd = torch.from_numpy(v.reshape(T, -1).view(np.int16)).cuda()
+    qd = torch.from_numpy(q.view(np.int16)).cuda()
+    shapes = [[19456], [19457], [4097, 15359], [4097, 15360], [500, 2], [40000], [9999], [20000, 20000]]
+    cus = [np.concatenate([[0], np.cumsum(l)]).astype(np.int32) for l in shapes]
+    ws = torch.zeros(max(ap.apack_decode_workspace_size(cu, 28, 4) for cu in cus), dtype=torch.uint8, device="cuda")
+    for cu in cus + cus[::-1]:
+        B = len(cu) - 1
+        out = torch.full((B, 28, 128), float("nan"), dtype=torch.float32, device="cuda")
+        ap.apack_decode_attention(cu, qd, kd, vd, 4 * 256, 28, 4, out, ws)
+        torch.cuda.synchronize()
+        assert ap.apack_device_error(ws) == ap.APACK_OK
+        n = int(cu[-1])
+        check(out.cpu().numpy(), oracle.decode_attention(q[:B], k[:n], v[:n], cu, 28, 4))
+
+
 RANDOM_HEADS = [(28, 4), (16, 2), (12, 4), (32, 4), (8, 2), (8, 8), (8, 1), (4, 4)]
 
 
