@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(32 * WARPS)
   __shared__ float2 wml[WARPS];
   pdl_wait_and_release();                   // the chunk kernel's partials are complete and visible
   const int s = blockIdx.x / plan.hq, hh = blockIdx.x % plan.hq;
-  if (hh == 0 && threadIdx.x == 0) claims[s] = 0u;
+  if (plan.claimed && hh == 0 && threadIdx.x < (1 << plan.split_log))
+    claims[(s << plan.split_log) + threadIdx.x] = 0u;
   const DecSeq &sq = plan.seq[s];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
@@ -521,6 +522,15 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     // 500 tokens 12.3 -> 7.9 us.
     P.split_log = 0;
     while ((num_kv_heads >> P.split_log) % 2 == 0 && (chunks << (P.split_log + 1)) <= device_sm_count()) ++P.split_log;
+    P.claimed = tc && P.split_log == 0;
+    // One cache whose chunks still leave SMs idle (whole 128-key tiles: 79 chunks of 256 keys for 20,000
+    // tokens): one more split, with as many CTAs as there are SMs; the claims deal the stages.  16/2 heads:
+    // 13.3 -> 11.6 us for 20,000 tokens, 15.9 -> 14.5 us for 40,000, 18.7 -> 17.7 us for 60,000.
+    if (tc && num_seqs == 1 && (num_kv_heads >> P.split_log) % 2 == 0 && 10 * (chunks << P.split_log) < 9 * device_sm_count()) {
+      ++P.split_log;
+      P.claimed = 1;
+      P.seq[0].nchunks = chunks = P.total_chunks = std::min(chunks, std::max(1, device_sm_count() >> P.split_log));
+    }
     float *op = opart + chunk_base * num_q_heads * 128;
     float2 *mp = mlpart + chunk_base * num_q_heads;
     const uint16_t *qs = q16 + static_cast<int64_t>(s0) * num_q_heads * 128;

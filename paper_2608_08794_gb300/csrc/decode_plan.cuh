@@ -15,6 +15,7 @@ struct DecSeq {
 struct DecPlan {
   int32_t nseq, hq, hkv, group, chunk;   // chunk: keys per CTA, a multiple of the kernel's tile
   int32_t total_chunks;
+  int32_t claimed;                       // tensor-core path: the stages are claimed (else: each CTA its own)
   int32_t split_log;                     // log2 of the CTAs per chunk, each with hkv >> split_log KV heads
   float scale2;                          // log2(e) / sqrt(128)
   DecSeq seq[kSeqsPerLaunch];
@@ -27,8 +28,9 @@ __device__ __forceinline__ int find_chunk_seq(const DecPlan &p, int c) {
 }
 
 // Tensor-core chunk kernel (decode_tc.cu): Hkv = 2 or 4, at most 8 query heads per KV head.
-// With split_log 0 the CTAs of sequence i claim its 128-key stages from claims[i] (zero before the launch;
-// the combine kernel zeroes it again); with more, every CTA has the stages of its chunk and heads.  A CTA
+// With `claimed` the CTAs of sequence i and heads j claim their 128-key stages from
+// claims[(i << split_log) + j] (zero before the launch; the combine kernel zeroes them again); without, every
+// CTA has the stages of its chunk and heads.  A CTA
 // writes one partial per query head of its heads, in the layout of the CUDA-core kernel's chunk partials.
 // grid: total_chunks << split_log.
 cudaError_t launch_decode_tc(int grid, cudaStream_t stream, const CUtensorMap &kmap, const CUtensorMap &vmap,

@@ -214,14 +214,17 @@ __global__ void __launch_bounds__(kDThreads, 1)
       // a CTA's first two units are its own (c and n + c of the sequence's n CTAs), the rest are claimed;
       // claims run two stages ahead of the loads (an atomic's round trip is about a stage's time); one
       // thread's claims on one counter return increasing units
-      unsigned int *claim = claims + s;
+      unsigned int *claim = claims + ((s << plan.split_log) + blockIdx.x - (c << plan.split_log));
       const int rank = c - sq.chunk_begin, own = 2 * sq.nchunks;
-      const bool claimed = plan.split_log == 0;
-      const int tile0 = rank * (plan.chunk / kDM);          // split: the chunk's tiles, this CTA's heads
-      const int mine = min(plan.chunk / kDM, units / HKV - tile0) * heads;
-      auto unit_of = [&](int n) { return n < mine ? (tile0 + n / heads) * HKV + h0 + n % heads : units; };
-      int next = claimed ? rank : unit_of(0);                   // stage 0's unit
-      int next2 = claimed ? sq.nchunks + rank : unit_of(1);     // stage 1's
+      const bool claimed = plan.claimed;
+      // claim x is stage base + x of this CTA's heads (heads = 1 << lg): of the sequence in the order of
+      // the claims, or of the chunk's tiles
+      const int lg = (HKV == 4 ? 2 : 1) - plan.split_log;
+      const int tile0 = claimed ? 0 : rank * (plan.chunk / kDM);
+      const int tiles = claimed ? units / HKV : min(plan.chunk / kDM, units / HKV - tile0);
+      const unsigned limit = static_cast<unsigned>(tiles << lg);
+      int next = claimed ? rank : 0;                        // stage 0's claim
+      int next2 = claimed ? sq.nchunks + rank : 1;          // stage 1's
       int unit[2] = {0, 0};                       // units of the last two claimed stages (by n & 1)
       int n_end = -1;                             // the number of claimed stages, once known
       int last = -1;                              // the last item issued with a load
@@ -235,16 +238,16 @@ __global__ void __launch_bounds__(kDThreads, 1)
         const int slot = i % kDSlots;
         if (!is_v) {
           // publish stage n's record (its unit, or the end of the claims) before its K load
-          const int u = next;
           const int r = n % kDInfo;
-          if (static_cast<unsigned>(u) >= static_cast<unsigned>(units)) {   // a counter left dirty ends the claims too
+          if (static_cast<unsigned>(next) >= limit) {   // a counter left dirty ends the claims too
             bars->info[r] = -1;
             mbar_arrive(&bars->info_full[r]);
             n_end = n;
             continue;                              // no load: V(n - 1) is the last item
           }
+          const int u = (tile0 + (next >> lg)) * HKV + h0 + (next & (heads - 1));
           next = next2;
-          next2 = claimed ? own + static_cast<int>(atomicAdd(claim, 1u)) : unit_of(n + 2);   // stage n + 2's unit
+          next2 = claimed ? own + static_cast<int>(atomicAdd(claim, 1u)) : n + 2;   // stage n + 2's claim
           unit[n & 1] = u;
           bars->info[r] = u;
           mbar_arrive(&bars->info_full[r]);

@@ -86,6 +86,7 @@ def test_decode_attention_matches_oracle(ap, lens, hq, hkv):
 @pytest.mark.parametrize("hq,hkv", [(28, 4), (8, 1), (5, 1), (8, 8), (16, 8), (24, 8), (32, 8)])
 @pytest.mark.parametrize("lens", [
     [128 * 152],                    # one tile per chunk: as many chunks as the wide combine merges in one round
+    [20000],                        # 79 chunks of 256 keys: claims per share of the heads
     [128 * 40], [128 * 41 - 1],     # 40 chunks, the most of the narrow combine's rounds, and 41
     [1, 127, 129, 2, 128 * 3],      # CTAs whose second own unit lies past the sequence
     [100 + 61 * i for i in range(48)],   # a last chunk per sequence would not fit one CTA per SM
