@@ -74,6 +74,27 @@ def test_frame_alignment_matches_oracle(ap, F, tpf, na, dim, window, tau):
     assert c.tobytes() == again[0].tobytes() and s.tobytes() == again[1].tobytes()
 
 
+@pytest.mark.parametrize("F,tpf,na,dim,window,tau", [
+    (457, 25, 460, 2048, 3, 0.0),     # runs of 4 frames on 152 SMs, the last of one frame
+    (458, 12, 458, 4096, 3, 0.999),   # the widest rows of a run; the last run of two frames
+    (608, 95, 700, 520, 3, 0.999),    # 31 rows a ring stage
+    (761, 72, 9000, 512, 5, 0.999),   # runs of 6, window 5
+    (457, 3, 5000, 72, 3, 0.0),       # too few bytes a run: one CTA per frame
+])
+def test_frame_alignment_runs_of_frames(ap, F, tpf, na, dim, window, tau):
+    from synth.gen import f32_to_bf16_bits
+    rng = np.random.default_rng(F + dim)
+    vis, aud = (f32_to_bf16_bits(rng.standard_normal((n, dim), dtype=np.float32)) for n in (F * tpf, na))
+    c, s, dn, cb = run(ap, vis, aud, F, tpf, dim, window, tau, 0.9)
+    ref = oracle.frame_alignment(vis, aud, F, tpf, window=window, tau=tau, beta=0.9)
+    np.testing.assert_allclose(c, ref["c"], atol=TOL, rtol=0)
+    np.testing.assert_allclose(dn, ref["dnorm"], atol=TOL, rtol=0)
+    np.testing.assert_allclose(s, ref["s"], atol=TOL, rtol=0)
+    assert cb == pytest.approx(ref["cbar"], abs=TOL)
+    again = run(ap, vis, aud, F, tpf, dim, window, tau, 0.9)
+    assert c.tobytes() == again[0].tobytes() and s.tobytes() == again[1].tobytes()
+
+
 def test_frame_alignment_two_and_a_half_minute_clip(ap):
     # 300 frames of 100 visual tokens, 25 audio tokens per second at 2 fps, 7B hidden size
     F, tpf, na, dim = 300, 100, 3750, 3584
