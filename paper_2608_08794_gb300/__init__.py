@@ -74,13 +74,13 @@ def _load():
         raise ImportError(f"libapack.so is not built ({LIB_PATH}); run __graft_entry__.build()")
     lib = ctypes.CDLL(LIB_PATH)
     P, I32, I64, SZ, VP = ctypes.POINTER, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t, ctypes.c_void_p
-    PI32 = P(I32)
+    PI32 = VP                     # host arrays go in as plain addresses (see _host)
     lib.apack_workspace_size.argtypes = [P(apack_seqs), P(SZ)]
-    lib.apack_keep_counts.argtypes = [P(apack_seqs), P(ctypes.c_float), I32, PI32, PI32]
+    lib.apack_keep_counts.argtypes = [P(apack_seqs), VP, I32, PI32, PI32]
     lib.apack_score.argtypes = [P(apack_seqs), VP, VP, I64, VP, VP, SZ, VP]
-    lib.apack_select.argtypes = [P(apack_seqs), VP, P(ctypes.c_float), PI32, I32, VP, VP, VP, VP, VP, SZ, VP]
+    lib.apack_select.argtypes = [P(apack_seqs), VP, VP, PI32, I32, VP, VP, VP, VP, VP, SZ, VP]
     lib.apack_compact.argtypes = [VP, I64, P(apack_plane), I32, VP, VP]
-    lib.apack_prune_step.argtypes = [P(apack_seqs), I32, I32, VP, VP, VP, I64, VP, I64, P(ctypes.c_float), PI32,
+    lib.apack_prune_step.argtypes = [P(apack_seqs), I32, I32, VP, VP, VP, I64, VP, I64, VP, PI32,
                                      I32, VP, VP, I64, VP, P(apack_plane), I32, VP, VP, PI32, VP, VP, VP, SZ,
                                      P(VP), VP]
     lib.apack_device_error.argtypes = [VP, VP, PI32, I32]
@@ -119,21 +119,43 @@ def _check(status, where):
 
 
 def _ptr(t):
-    """Device pointer of a torch tensor (or None -> NULL)."""
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    """Device address of a torch tensor (or None -> NULL)."""
+    return None if t is None else t.data_ptr()
+
+
+def _current_stream():
+    """The current device's current stream, as an address.  torch.cuda.current_stream() builds a
+    Stream object on every call; its raw handle is the same."""
+    import torch
+    if torch.cuda.is_initialized():
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return _current_stream()
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _i32(a):
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
+
+
+def _f32(a):
+    return np.ascontiguousarray(np.asarray(a, dtype=np.float32))
+
+
+def _host(a):
+    """Address of a contiguous host array (or None -> NULL); the caller keeps the array alive."""
+    return None if a is None else a.ctypes.data
+
+
+def _planes(planes):
+    return (apack_plane * len(planes))(*planes) if len(planes) else None
 
 
 class Seqs:
@@ -185,9 +207,7 @@ def apack_keep_counts(seqs, keep_ratio, select_mode=APACK_SELECT_PER_MODALITY):
     r = np.ascontiguousarray(np.asarray(keep_ratio, dtype=np.float32).reshape(seqs.num_seqs, 2))
     k = np.zeros((seqs.num_seqs, 2), np.int32)
     cu = np.zeros(seqs.num_seqs + 1, np.int32)
-    I32P = ctypes.POINTER(ctypes.c_int32)
-    _check(_lib.apack_keep_counts(seqs.ref(), r.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), select_mode,
-                                  k.ctypes.data_as(I32P), cu.ctypes.data_as(I32P)), "apack_keep_counts")
+    _check(_lib.apack_keep_counts(seqs.ref(), _host(r), select_mode, _host(k), _host(cu)), "apack_keep_counts")
     return k, cu
 
 
@@ -199,12 +219,9 @@ def apack_score(seqs, q, k, k_token_stride, scores, ws, stream=None):
 def apack_select(seqs, scores, keep_count, keep_idx, ws, select_mode=APACK_SELECT_PER_MODALITY,
                  modality_out=None, dst_of_src=None, new_cu_seqlens=None, stream=None, keep_ratio=None):
     """keep_count: [B, 2] counts, or None with keep_ratio [B, 2] (ratios 1-P of Eq. inner)."""
-    kc = None if keep_count is None else _i32(keep_count).reshape(-1)
-    kr = None if keep_ratio is None else np.ascontiguousarray(np.asarray(keep_ratio, np.float32).reshape(-1))
-    _check(_lib.apack_select(seqs.ref(), _ptr(scores),
-                             None if kr is None else kr.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
-                             None if kc is None else kc.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                             select_mode, _ptr(keep_idx), _ptr(modality_out), _ptr(dst_of_src),
+    kc = None if keep_count is None else _i32(keep_count)
+    kr = None if keep_ratio is None else _f32(keep_ratio)
+    _check(_lib.apack_select(seqs.ref(), _ptr(scores), _host(kr), _host(kc), select_mode, _ptr(keep_idx), _ptr(modality_out), _ptr(dst_of_src),
                              _ptr(new_cu_seqlens), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)),
            "apack_select")
 
@@ -220,8 +237,7 @@ def make_plane(src, dst, row_bytes, num_planes=1, src_plane_stride=0, dst_plane_
 
 
 def apack_compact(keep_idx, n_out, planes, ws=None, stream=None):
-    arr = (apack_plane * max(1, len(planes)))(*planes)
-    _check(_lib.apack_compact(_ptr(keep_idx), int(n_out), arr, len(planes), _ptr(ws), _stream(stream)),
+    _check(_lib.apack_compact(_ptr(keep_idx), int(n_out), _planes(planes), len(planes), _ptr(ws), _stream(stream)),
            "apack_compact")
 
 
@@ -231,13 +247,11 @@ def apack_prune_step(seqs, layer, num_layers, q, k_cache, v_cache, kv_layer_stri
                      keep_idx=None, new_cu_seqlens=None, scores=None, ws=None, stage_events=None, stream=None):
     """One pruning step; returns the new packed offsets (host numpy [B+1])."""
     B = seqs.num_seqs
-    I32P = ctypes.POINTER(ctypes.c_int32)
     ratio = None
     if keep_ratio is not None:
         ratio = np.ascontiguousarray(np.asarray(keep_ratio, dtype=np.float32).reshape(B, 2))
-    kc = None if keep_count is None else _i32(keep_count).reshape(-1)
+    kc = None if keep_count is None else _i32(keep_count)
     new_cu = np.zeros(B + 1, np.int32)
-    arr = (apack_plane * max(1, len(extra_planes)))(*extra_planes)
     ev = None
     if stage_events is not None:
         handles = [e.cuda_event if hasattr(e, "cuda_event") else e for e in stage_events]
@@ -246,11 +260,9 @@ def apack_prune_step(seqs, layer, num_layers, q, k_cache, v_cache, kv_layer_stri
         ev = (ctypes.c_void_p * 4)(*handles)
     st = _lib.apack_prune_step(
         seqs.ref(), int(layer), int(num_layers), _ptr(q), _ptr(k_cache), _ptr(v_cache), int(kv_layer_stride),
-        _ptr(hidden), int(hidden_dim),
-        None if ratio is None else ratio.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
-        None if kc is None else kc.ctypes.data_as(I32P), select_mode, _ptr(k_out), _ptr(v_out),
-        int(kv_out_layer_stride), _ptr(hidden_out), arr, len(extra_planes), _ptr(modality_out), _ptr(keep_idx),
-        new_cu.ctypes.data_as(I32P), _ptr(new_cu_seqlens), _ptr(scores), _ptr(ws),
+        _ptr(hidden), int(hidden_dim), _host(ratio), _host(kc), select_mode, _ptr(k_out), _ptr(v_out),
+        int(kv_out_layer_stride), _ptr(hidden_out), _planes(extra_planes), len(extra_planes), _ptr(modality_out),
+        _ptr(keep_idx), _host(new_cu), _ptr(new_cu_seqlens), _ptr(scores), _ptr(ws),
         0 if ws is None else ws.numel() * ws.element_size(), ev, _stream(stream))
     _check(st, "apack_prune_step")
     return new_cu
@@ -382,7 +394,7 @@ def apack_frame_alignment(visual, audio, n_frames, tokens_per_frame, n_audio, di
 def apack_decode_workspace_size(cu_seqlens, num_q_heads, num_kv_heads):
     cu = _i32(cu_seqlens)
     n = ctypes.c_size_t(0)
-    _check(_lib.apack_decode_workspace_size(len(cu) - 1, cu.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), int(num_q_heads),
+    _check(_lib.apack_decode_workspace_size(len(cu) - 1, _host(cu), int(num_q_heads),
                                             int(num_kv_heads), ctypes.byref(n)), "apack_decode_workspace_size")
     return n.value
 
@@ -390,7 +402,7 @@ def apack_decode_workspace_size(cu_seqlens, num_q_heads, num_kv_heads):
 def apack_decode_attention(cu_seqlens, q, k, v, kv_token_stride, num_q_heads, num_kv_heads, out, ws, stream=None):
     """Attention of one decode token per sequence over its KV cache (Sec. 3.2)."""
     cu = _i32(cu_seqlens)
-    _check(_lib.apack_decode_attention(len(cu) - 1, cu.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _ptr(q), _ptr(k), _ptr(v),
+    _check(_lib.apack_decode_attention(len(cu) - 1, _host(cu), _ptr(q), _ptr(k), _ptr(v),
                                        int(kv_token_stride), int(num_q_heads), int(num_kv_heads), _ptr(out),
                                        _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)),
            "apack_decode_attention")

@@ -231,8 +231,10 @@ apack_status apack_select(const apack_seqs *seqs, const float *scores, const flo
 apack_status apack_compact(const int32_t *keep_idx, int64_t n_out, const apack_plane *planes_h, int32_t num_groups,
                            void *ws, void *stream) {
   if (ws && (reinterpret_cast<uintptr_t>(ws) & 255)) return APACK_EINVAL;
-  return run_compact(keep_idx, n_out, planes_h, num_groups, static_cast<DeviceError *>(ws),
-                     static_cast<cudaStream_t>(stream));
+  const CompactPlanPtr plan(new_compact_plan());
+  if (!plan) return APACK_ECUDA;
+  const apack_status st = plan_compact(*plan, keep_idx, n_out, planes_h, num_groups, static_cast<DeviceError *>(ws));
+  return st == APACK_OK ? launch_compact(*plan, static_cast<cudaStream_t>(stream)) : st;
 }
 
 apack_status apack_prune_step(const apack_seqs *seqs, int32_t layer, int32_t num_layers, const void *q,
@@ -292,7 +294,9 @@ apack_status apack_prune_step(const apack_seqs *seqs, int32_t layer, int32_t num
   for (int i = 0; i < num_extra; ++i) planes.push_back(extra_planes_h[i]);
   DeviceError *err = reinterpret_cast<DeviceError *>(static_cast<uint8_t *>(ws) + workspace_layout(seqs).err_off);
   // every argument of the compaction is checked before the first launch of the step
-  st = run_compact(keep_idx, n_out, planes.data(), static_cast<int32_t>(planes.size()), err, s, true);
+  const CompactPlanPtr compact(new_compact_plan());
+  if (!compact) return APACK_ECUDA;
+  st = plan_compact(*compact, keep_idx, n_out, planes.data(), static_cast<int32_t>(planes.size()), err);
   if (st != APACK_OK) return st;
   auto mark = [&](int i) {
     if (stage_events_h && stage_events_h[i]) cudaEventRecord(static_cast<cudaEvent_t>(stage_events_h[i]), s);
@@ -304,7 +308,7 @@ apack_status apack_prune_step(const apack_seqs *seqs, int32_t layer, int32_t num
   st = run_select(seqs, scores, counts.data(), select_mode, keep_idx, modality_out, nullptr, new_cu_seqlens, ws, s);
   if (st != APACK_OK) return st;
   mark(2);
-  st = run_compact(keep_idx, n_out, planes.data(), static_cast<int32_t>(planes.size()), err, s);
+  st = launch_compact(*compact, s);
   if (st != APACK_OK) return st;
   mark(3);
   return APACK_OK;

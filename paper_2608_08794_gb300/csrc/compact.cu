@@ -9,6 +9,8 @@
 //  - a source in pinned host memory: the zero-copy gather below;
 //  - rows that are not 16-byte multiples (or misaligned): the narrow kernel below, one thread
 //    per row.
+#include <new>
+
 #include "compact_plan.cuh"
 
 namespace apack {
@@ -121,19 +123,32 @@ bool ranges_overlap(const apack_plane &p, int64_t n_rows_src, int64_t n_out) {
 
 }  // namespace
 
-apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_plane *planes, int32_t num_groups,
-                         DeviceError *err, cudaStream_t stream, bool check_only) {
+class CompactPlan {
+ public:
+  const int32_t *keep_idx = nullptr;
+  int64_t n_out = 0;
+  DeviceError *err = nullptr;
+  TmaPlan tp{}, ip{};                    // out-of-place groups, in-place groups
+  uint32_t in_blocks = 0;
+  apack_plane narrow[kMaxGroups * 4], host_groups[kMaxGroups * 4];
+  int n_narrow = 0, n_host = 0;
+};
+
+CompactPlan *new_compact_plan() { return new (std::nothrow) CompactPlan; }
+void CompactPlanDelete::operator()(CompactPlan *p) const { delete p; }
+
+apack_status plan_compact(CompactPlan &plan, const int32_t *keep_idx, int64_t n_out, const apack_plane *planes,
+                          int32_t num_groups, DeviceError *err) {
   if (n_out < 0 || num_groups < 0 || (num_groups > 0 && !planes)) return APACK_EINVAL;
   if (n_out == 0 || num_groups == 0) return APACK_OK;
   if (!keep_idx || n_out > INT32_MAX) return APACK_EINVAL;
   // validate and plan every group before anything touches the device
-  TmaPlan tp{}, ip{};           // out-of-place groups, in-place groups
+  plan.keep_idx = keep_idx;
+  plan.n_out = n_out;
+  plan.err = err;
+  TmaPlan &tp = plan.tp, &ip = plan.ip;
   tp.n_out = ip.n_out = static_cast<uint32_t>(n_out);
   uint64_t items = 0, in_items = 0;
-  int narrow[kMaxGroups * 4];
-  int n_narrow = 0;
-  apack_plane host_groups[kMaxGroups * 4];
-  int n_host = 0;
   for (int i = 0; i < num_groups; ++i) {
     const apack_plane &p = planes[i];
     if (p.num_planes < 0 || p.row_bytes < 0) return APACK_EINVAL;
@@ -145,13 +160,13 @@ apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_pla
     if (const void *hs = host_source(p.src)) {
       // pinned host source: zero-copy gather (destination in device memory, never in place)
       if (p.src == p.dst || host_source(p.dst)) return APACK_EINVAL;
-      if (n_host == kMaxGroups * 4) return APACK_EINVAL;
+      if (plan.n_host == kMaxGroups * 4) return APACK_EINVAL;
       if (widest_unit(p) == 16 && static_cast<int64_t>(p.num_planes) * n_out * (p.row_bytes / 16) >
                                       0x7FFFFFFFLL * kHostPiecesPerCta)
         return APACK_EUNSUPPORTED;                  // beyond one launch's grid
-      host_groups[n_host] = p;
-      host_groups[n_host].src = hs;
-      ++n_host;
+      plan.host_groups[plan.n_host] = p;
+      plan.host_groups[plan.n_host].src = hs;
+      ++plan.n_host;
       continue;
     }
     if (p.src == p.dst) {
@@ -183,18 +198,19 @@ apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_pla
       cnt += static_cast<uint64_t>(g.chunks_per_plane) * p.num_planes;
       if (cnt > 0x7FFFFFFFull) return APACK_EINVAL;
     } else {
-      if (n_narrow == kMaxGroups * 4) return APACK_EINVAL;
-      narrow[n_narrow++] = i;
+      if (plan.n_narrow == kMaxGroups * 4) return APACK_EINVAL;
+      plan.narrow[plan.n_narrow++] = p;
     }
   }
-  uint32_t in_blocks = 0;
-  if (ip.ngroups > 0) {
-    const apack_status st = plan_inplace(ip, in_items, &in_blocks);
-    if (st != APACK_OK) return st;
-  }
-  if (check_only) return APACK_OK;
-  for (int k = 0; k < n_host; ++k) {
-    const apack_plane &p = host_groups[k];
+  tp.total_items = static_cast<uint32_t>(items);
+  return ip.ngroups > 0 ? plan_inplace(ip, in_items, &plan.in_blocks) : APACK_OK;
+}
+
+apack_status launch_compact(const CompactPlan &plan, cudaStream_t stream) {
+  const int32_t *keep_idx = plan.keep_idx;
+  const int64_t n_out = plan.n_out;
+  for (int k = 0; k < plan.n_host; ++k) {
+    const apack_plane &p = plan.host_groups[k];
     if (widest_unit(p) == 16) {
       const int64_t n = static_cast<int64_t>(p.num_planes) * n_out * (p.row_bytes / 16);
       const int64_t blocks = (n + kHostPiecesPerCta - 1) / kHostPiecesPerCta;   // checked when planned
@@ -210,8 +226,8 @@ apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_pla
     count_launches(1);
     if (check_cuda(cudaGetLastError()) != APACK_OK) return APACK_ECUDA;
   }
-  for (int k = 0; k < n_narrow; ++k) {
-    const apack_plane &p = planes[narrow[k]];
+  for (int k = 0; k < plan.n_narrow; ++k) {
+    const apack_plane &p = plan.narrow[k];
     const int64_t n = static_cast<int64_t>(p.num_planes) * n_out;
     const int threads = 256;
     gather_narrow_kernel<<<static_cast<unsigned>((n + threads - 1) / threads), threads, 0, stream>>>(
@@ -220,11 +236,9 @@ apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_pla
     count_launches(1);
     if (check_cuda(cudaGetLastError()) != APACK_OK) return APACK_ECUDA;
   }
-  if (tp.ngroups > 0) {
-    tp.total_items = static_cast<uint32_t>(items);
-    if (launch_out_of_place(tp, keep_idx, err, stream) != APACK_OK) return APACK_ECUDA;
-  }
-  if (ip.ngroups > 0 && launch_inplace(ip, in_blocks, keep_idx, err, stream) != APACK_OK) return APACK_ECUDA;
+  if (plan.tp.ngroups > 0 && launch_out_of_place(plan.tp, keep_idx, plan.err, stream) != APACK_OK) return APACK_ECUDA;
+  if (plan.ip.ngroups > 0 && launch_inplace(plan.ip, plan.in_blocks, keep_idx, plan.err, stream) != APACK_OK)
+    return APACK_ECUDA;
   return APACK_OK;
 }
 

@@ -6,6 +6,7 @@
 #include <atomic>
 #include <cstddef>
 #include <cstdint>
+#include <memory>
 
 #include "apack.h"
 
@@ -129,10 +130,17 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
 apack_status run_select(const apack_seqs *seqs, const float *scores, const int32_t *keep_count_h, int32_t mode,
                         int32_t *keep_idx, uint8_t *modality_out, int32_t *dst_of_src, int32_t *new_cu_seqlens,
                         void *ws, cudaStream_t stream);
-// check_only: validate and plan every group, launch nothing (callers that launch other
-// kernels first check their compaction this way before any launch).
-apack_status run_compact(const int32_t *keep_idx, int64_t n_out, const apack_plane *planes, int32_t num_groups,
-                         DeviceError *err, cudaStream_t stream, bool check_only = false);
+// A checked and planned compaction, without its launches: callers that launch other kernels first plan
+// theirs before any launch (each source pointer is asked for its memory kind once).
+class CompactPlan;
+CompactPlan *new_compact_plan();
+struct CompactPlanDelete {
+  void operator()(CompactPlan *p) const;
+};
+using CompactPlanPtr = std::unique_ptr<CompactPlan, CompactPlanDelete>;
+apack_status plan_compact(CompactPlan &plan, const int32_t *keep_idx, int64_t n_out, const apack_plane *planes,
+                          int32_t num_groups, DeviceError *err);
+apack_status launch_compact(const CompactPlan &plan, cudaStream_t stream);
 // 3-D TMA map over a K slab [tokens][hkv][128] bf16 (token_stride bytes between tokens):
 // boxes of 64 features x 1 head x box_tokens tokens, 128-byte swizzle.
 bool make_kv_tile_map(CUtensorMap *map, const void *k, int hkv, int64_t tokens, int64_t token_stride,

@@ -20,7 +20,7 @@ struct StepPlan {
   apack_seqs seqs{};
   const void *k = nullptr, *v = nullptr, *hidden = nullptr;
   int64_t kv_layer_stride = 0;
-  std::vector<apack_plane> planes;     // the step's compaction groups
+  CompactPlanPtr compact;              // the step's compaction
 };
 
 apack_plane plane(const void *src, void *dst, int64_t src_ps, int64_t dst_ps, int64_t row, int32_t n) {
@@ -116,12 +116,15 @@ apack_status apack_prune_schedule(const apack_seqs *seqs, int32_t num_layers, co
       return APACK_EINVAL;
     // compaction: K/V of layers [l_i, L), hidden, extra planes, in one launch
     if (sp.num_extra < 0 || (sp.num_extra > 0 && !sp.extra_planes_h)) return APACK_EINVAL;
-    p.planes.reserve(3 + static_cast<size_t>(sp.num_extra));
-    p.planes.push_back(plane(p.k, sp.k_out, p.kv_layer_stride, sp.kv_out_layer_stride, row, n_layers));
-    p.planes.push_back(plane(p.v, sp.v_out, p.kv_layer_stride, sp.kv_out_layer_stride, row, n_layers));
-    if (p.hidden) p.planes.push_back(plane(p.hidden, sp.hidden_out, 0, 0, hidden_dim * 2, 1));
-    for (int e = 0; e < sp.num_extra; ++e) p.planes.push_back(sp.extra_planes_h[e]);
-    st = run_compact(sp.keep_idx, n_out, p.planes.data(), static_cast<int32_t>(p.planes.size()), err, nullptr, true);
+    std::vector<apack_plane> planes;
+    planes.reserve(3 + static_cast<size_t>(sp.num_extra));
+    planes.push_back(plane(p.k, sp.k_out, p.kv_layer_stride, sp.kv_out_layer_stride, row, n_layers));
+    planes.push_back(plane(p.v, sp.v_out, p.kv_layer_stride, sp.kv_out_layer_stride, row, n_layers));
+    if (p.hidden) planes.push_back(plane(p.hidden, sp.hidden_out, 0, 0, hidden_dim * 2, 1));
+    for (int e = 0; e < sp.num_extra; ++e) planes.push_back(sp.extra_planes_h[e]);
+    p.compact.reset(new_compact_plan());
+    if (!p.compact) return APACK_ECUDA;
+    st = plan_compact(*p.compact, sp.keep_idx, n_out, planes.data(), static_cast<int32_t>(planes.size()), err);
     if (st != APACK_OK) return st;
   }
 
@@ -141,8 +144,7 @@ apack_status apack_prune_schedule(const apack_seqs *seqs, int32_t num_layers, co
                     sp.new_cu_seqlens, ws, M);
     if (st != APACK_OK) return st;
     mark(i, 2);
-    st = run_compact(sp.keep_idx, sp.new_cu_seqlens_h[B], p.planes.data(), static_cast<int32_t>(p.planes.size()),
-                     err, M);
+    st = launch_compact(*p.compact, M);
     if (st != APACK_OK) return st;
     mark(i, 3);
   }
