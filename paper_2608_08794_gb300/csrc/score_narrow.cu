@@ -35,6 +35,14 @@ constexpr int kPartTokens = 64;        // a sequence has at most one partial per
 // Rows times partials of a sequence up to which every CTA of the final kernel merges the partials by
 // itself instead of a kernel of its own before it.
 constexpr int kMergeInside = 16384;
+// Keys read as the first to leave the 129 MB L2, for the logits to stay in it until the final kernel: where
+// the keys are more than the first figure (below it they may stay for what reads them next) and the
+// logits less than the second. 28/4 heads, normal -> first to leave: keys 98 MB 29.1 -> 27.9 us, 132 MB
+// 36.7 -> 34.7 us and with four query rows 64.4 -> 56.4 us, 488 MB 120.5 -> 114.5 us; 16 sequences, 262 MB
+// and 60 MB of logits 104.2 -> 96.5 us; but 66 MB 19.7 -> 19.5 us, and 293 MB beside 134 MB of logits
+// 127.8 -> 129.9 us.
+constexpr int64_t kStreamKeyBytes = 96 << 20;
+constexpr int64_t kStreamLogitBytes = 100 << 20;
 constexpr int kLogitPad = 64;          // logit row stride: the key count rounded up to this
 
 __device__ __forceinline__ bool is_mm(uint8_t m) { return m == APACK_MOD_AUDIO || m == APACK_MOD_VISUAL; }
@@ -385,11 +393,14 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       return std::min<int64_t>((stages_of(b) + chunk - 1) / chunk, (len + kPartTokens - 1) / kPartTokens);
     };
     const int64_t sms = device_sm_count();
-    int64_t all_stages = 0, max_stages = 1;
+    int64_t all_stages = 0, max_stages = 1, logit_bytes = 0;
     for (int i = 0; i < ns; ++i) {
+      const int64_t len = seqs->cu_seqlens_h[s0 + i + 1] - seqs->cu_seqlens_h[s0 + i];
+      logit_bytes += len * hq * (seqs->cu_qlens_h[s0 + i + 1] - seqs->cu_qlens_h[s0 + i]) * 4;
       all_stages += stages_of(s0 + i);
       max_stages = std::max(max_stages, stages_of(s0 + i));
     }
+    P.stream_keys = all_stages * (128 * 256) > kStreamKeyBytes && logit_bytes < kStreamLogitBytes;
     int64_t chunk = std::max<int64_t>(1, (all_stages + sms - 1) / sms);
     for (; chunk < max_stages; chunk += std::max<int64_t>(1, chunk / 32)) {
       int64_t ctas = 0;

@@ -152,14 +152,16 @@ __global__ void __launch_bounds__(TcLayout<HKV, NR>::kThreads, 1)
     tc_fence_before();
   }
   pdl_wait_and_release();   // the set-up above runs beside the previous launch; q and K are read below
+  // many keys are read as the first to leave L2, so that the logits stay for the final kernel
+  const uint64_t policy = plan.stream_keys ? l2_evict_first() : l2_evict_normal();
   // stage n of this CTA: unit u0 + n = tile * HKV + head
   auto issue_load = [&](int n) {
     const int slot = n % kStages, t = (u0 + n) / HKV, h = (u0 + n) % HKV;
     uint8_t *dst = ring + slot * kTcStageBytes;
     const int key0 = sq.t0 + t * kTcM;
     mbar_arrive_expect_tx(&bars->k_full[slot], kTcStageBytes);
-    tma_load_3d(dst, &kmap, &bars->k_full[slot], 0, h, key0);
-    tma_load_3d(dst + kTcHalf, &kmap, &bars->k_full[slot], 64, h, key0);
+    tma_load_3d_hint(dst, &kmap, &bars->k_full[slot], 0, h, key0, policy);
+    tma_load_3d_hint(dst + kTcHalf, &kmap, &bars->k_full[slot], 64, h, key0, policy);
   };
   const int first = min(nstage, kStages);
   if (threadIdx.x == 0)
