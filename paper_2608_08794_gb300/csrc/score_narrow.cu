@@ -13,12 +13,13 @@
 //                     with the group's query rows held in shared memory;
 //   final kernel:   the row normalisers lse2 from the CTA partials, then one thread per key sums
 //                   exp2(x log2(e)/sqrt(D) - lse2) over all logit rows in a fixed order and scales
-//                   by 1/(Hq n_q).  When a sequence has many partials (kMergeInside) a merge kernel
+//                   by 1/(Hq n_q).  Above 32 rows or with many partials (kMergeInside) a merge kernel
 //                   computes lse2 first.
 // The logits of the 10-minute 7B sequence with one query row take 15 MB and stay
 // in L2 between the first and the last kernel.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "narrow_plan.cuh"
@@ -32,8 +33,12 @@ constexpr int kThreads = 256;          // keys per CTA (general logits kernel)
 constexpr int kWarps = kThreads / 32;
 constexpr int kFinalThreads = 512;     // threads per CTA (final kernel)
 constexpr int kPartTokens = 64;        // a sequence has at most one partial per this many keys (sizes the workspace)
-// Rows times partials of a sequence up to which every CTA of the final kernel merges the partials by
-// itself instead of a kernel of its own before it.
+// Rows of a sequence, and rows times its partials, up to which every CTA of the final kernel merges the
+// partials by itself instead of a kernel of its own before it: one round of its warps.  Inside / a kernel of
+// its own, 28/4 heads: 28 rows of 8,400 keys 9.4 / 9.9 us, 16 sequences of 8,400 33.4 / 35.2; 56 rows of
+// 4,000 keys 11.2 / 10.6, 67,500 27.7 / 25.0; 84 rows of 67,500 36.1 / 31.8; but 56 rows of 40 sequences of
+// 600 keys 18.9 / 20.7.
+constexpr int kMergeRows = 32;
 constexpr int kMergeInside = 16384;
 // Keys read as the first to leave the 129 MB L2, for the logits to stay in it until the final kernel: where
 // the keys are more than the first figure (below it they may stay for what reads them next) and the
@@ -218,14 +223,59 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// One warp merges a row's partials p[0..n): the first 32 kHold in registers, so that their loads can be
+// issued before the work of another row.  Returns lse2; +inf where no key is in the denominator.
+constexpr int kHold = 5;
+
+__device__ __forceinline__ void load_parts(const float2 *p, int n, int lane, float2 (&v)[kHold]) {
+#pragma unroll
+  for (int i = 0; i < kHold; ++i) v[i] = lane + 32 * i < n ? p[lane + 32 * i] : make_float2(-INFINITY, 0.f);
+}
+
+__device__ __forceinline__ float merge_parts(const float2 *p, int n, int lane, const float2 (&v)[kHold]) {
+  float m = v[0].x, sum = 0.f;
+#pragma unroll
+  for (int i = 1; i < kHold; ++i) m = fmaxf(m, v[i].x);
+  for (int c = lane + 32 * kHold; c < n; c += 32) m = fmaxf(m, p[c].x);
+  m = warp_max(m);
+  if (m != -INFINITY) {
+#pragma unroll
+    for (int i = 0; i < kHold; ++i) sum += v[i].y * exp2f(v[i].x - m);
+    for (int c = lane + 32 * kHold; c < n; c += 32) sum += p[c].y * exp2f(p[c].x - m);
+  }
+  sum = warp_sum(sum);
+  return m == -INFINITY ? INFINITY : m + log2f(sum);
+}
+
+// The merge with one warp per logit row, where no row has more than 32 kHold partials.  84 rows of each of
+// 40 sequences of 600 keys: 24.5 us for the whole call where a CTA per row took 34.5.
+__global__ void __launch_bounds__(kThreads)
+    score_narrow_merge_rows_kernel(const __grid_constant__ NarrowPlan plan, const float2 *__restrict__ part,
+                                   float *__restrict__ lse2, int rows_all) {
+  pdl_wait_and_release();
+  const int lane = threadIdx.x & 31, e = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (e >= rows_all) return;
+  int s = 0, acc = 0;
+  while (s + 1 < plan.nseq && acc + plan.seq[s].rows <= e) acc += plan.seq[s++].rows;
+  const NSeq &sq = plan.seq[s];
+  const int rho = e - acc;
+  const float2 *p = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
+  float2 v[kHold];
+  load_parts(p, sq.nparts, lane, v);
+  const float r = merge_parts(p, sq.nparts, lane, v);
+  if (lane == 0) lse2[sq.lse_base + rho] = r;
+}
+
 // One thread per key: I = sum over logit rows of exp2(x c2 - lse2) / (Hq n_q), x the stored dot
-// product.  MERGE: the CTA's warps first merge the sequence's partials into lse2, two rows per warp
-// and round, while the keys' own logits are in flight (a fixed order).  SPLIT threads share a key's
-// rows when there are more than 32 of them, so that a thread's loads stay one or two rounds.
-// Latency-bound (two L2 round trips and the launch): 8.5 us for 28 rows of 135,041 keys, where the
-// merge and final kernels took 10.3 us in two launches.
-template <bool MERGE, int SPLIT>
-__global__ void __launch_bounds__(kFinalThreads)
+// product.  MERGE (at most 32 rows): the CTA's warps first merge the sequence's partials into lse2
+// while the keys' own logits are in flight (a fixed order).  SPLIT threads share a key's rows, so that
+// a thread's loads stay a few rounds.  OCC: CTAs per SM; one where the grid is no more than that, with
+// the registers for all loads at once, else two within 64 registers.
+// Latency-bound (two or three L2 round trips and the launch).  The whole call with one CTA per SM / two:
+// 84 rows of 8,400 keys 11.4 / 12.0 us, 84 rows of 67,500 (264 CTAs) 29.8 / 29.3, 112 rows of 16 x 16,800
+// 108 / 101; 28 rows of 67,500 keys (132 CTAs) 18.9 / 20.1, of 135,041 35.7 / 34.7.
+template <bool MERGE, int SPLIT, int OCC>
+__global__ void __launch_bounds__(kFinalThreads, OCC)
     score_narrow_final_kernel(const __grid_constant__ NarrowPlan plan, const uint8_t *__restrict__ modality,
                               const float *__restrict__ logits, const float2 *__restrict__ part,
                               const float *__restrict__ lse2, float *__restrict__ scores) {
@@ -250,37 +300,23 @@ __global__ void __launch_bounds__(kFinalThreads)
   for (int u = 0; u < 32; ++u) raw[u] = (in && ra + u < rb) ? lp[static_cast<int64_t>(ra + u) * sq.lstride] : 0.f;
   if (MERGE) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // two rows per warp and round, the loads of both issued together; each row's first 160 partials
-    // are read once
-    constexpr int kHold = 5;
-    for (int r0 = warp; r0 < R; r0 += 2 * (kFinalThreads / 32)) {
-      float2 v[2][kHold];
+    constexpr int kAtOnce = OCC == 1 ? 2 : 1;            // rows of a warp whose loads are issued together
+#pragma unroll 1
+    for (int r0 = warp; r0 < R; r0 += kAtOnce * (kFinalThreads / 32)) {
+      float2 v[kAtOnce][kHold];
+      const float2 *p[kAtOnce];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < kAtOnce; ++k) {
         const int rho = r0 + k * (kFinalThreads / 32);
-        const float2 *p = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
-#pragma unroll
-        for (int i = 0; i < kHold; ++i)
-          v[k][i] = rho < R && lane + 32 * i < sq.nparts ? p[lane + 32 * i] : make_float2(-INFINITY, 0.f);
+        p[k] = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
+        load_parts(p[k], rho < R ? sq.nparts : 0, lane, v[k]);
       }
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < kAtOnce; ++k) {
         const int rho = r0 + k * (kFinalThreads / 32);
         if (rho >= R) break;                             // uniform over the warp
-        const float2 *p = part + sq.part_base + static_cast<int64_t>(rho) * sq.nparts;
-        float m = v[k][0].x, sum = 0.f;
-#pragma unroll
-        for (int i = 1; i < kHold; ++i) m = fmaxf(m, v[k][i].x);
-        for (int c = lane + 32 * kHold; c < sq.nparts; c += 32) m = fmaxf(m, p[c].x);
-        m = warp_max(m);
-        if (m != -INFINITY) {
-#pragma unroll
-          for (int i = 0; i < kHold; ++i) sum += v[k][i].y * exp2f(v[k][i].x - m);
-          for (int c = lane + 32 * kHold; c < sq.nparts; c += 32) sum += p[c].y * exp2f(p[c].x - m);
-        }
-        sum = warp_sum(sum);
-        // no key in the denominator: nothing is scored in this row
-        if (lane == 0) ls[rho] = m == -INFINITY ? -INFINITY : -(m + log2f(sum));
+        const float r = merge_parts(p[k], sq.nparts, lane, v[k]);
+        if (lane == 0) ls[rho] = -r;
       }
     }
   } else {
@@ -407,11 +443,28 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       for (int i = 0; i < ns; ++i) ctas += ctas_of(s0 + i, chunk);
       if (ctas <= sms) break;
     }
-    // the final kernel's threads per key: up to 32 rows each, then twice that
-    const int split = hq * (max_rg / G) <= 32 ? 1 : hq * (max_rg / G) <= 128 ? 2 : 4;
+    // The final kernel's threads per key: two above 32 rows and four above 128, so that a thread's loads stay
+    // a few rounds.  While all its CTAs still run at once, four above 64 rows (84 rows of 8,400 keys 13.65 ->
+    // 12.9 us); when there are more than two CTAs per SM the loads of other CTAs hide a thread's rounds, and
+    // one does up to 128 rows (112 rows of 135,041 keys 55.4 -> 51.9 us, 16 sequences of 16,800 keys 120.8 ->
+    // 108.3 us; at 264 CTAs, 67,500 keys, both 31.7 us).
+    auto final_ctas = [&](int per_key) {
+      int64_t n = 0;
+      for (int i = 0; i < ns; ++i)
+        n += (static_cast<int64_t>(seqs->cu_seqlens_h[s0 + i + 1] - seqs->cu_seqlens_h[s0 + i]) * per_key +
+              kFinalThreads - 1) / kFinalThreads;
+      return n;
+    };
+    const int seq_rows = hq * (max_rg / G);
+    const int split = seq_rows <= 32                              ? 1
+                      : seq_rows > 128                            ? 4
+                      : seq_rows > 64 && final_ctas(4) <= sms     ? 4
+                      : final_ctas(2) > 2 * sms                   ? 1
+                                                                  : 2;
     const int final_keys = kFinalThreads / split;
     int units = 0, units8 = 0, finals = 0, max_rows = 0;
     int64_t rows_all = 0, max_parts = 0;
+    int max_nparts = 0;
     for (int i = 0; i < ns; ++i) {
       const int b = s0 + i;
       NSeq &sq = P.seq[i];
@@ -442,6 +495,7 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       lse_base += sq.rows;
       rows_all += sq.rows;
       max_rows = sq.rows > max_rows ? sq.rows : max_rows;
+      max_nparts = std::max(max_nparts, sq.nparts);
       max_parts = std::max(max_parts, static_cast<int64_t>(sq.rows) * sq.nparts);
     }
     P.total_units = units;
@@ -469,16 +523,25 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
-    const bool inside = max_parts <= kMergeInside;
+    const bool inside = max_rows <= kMergeRows && max_parts <= kMergeInside;
     if (rows_all > 0 && !inside) {
-      if (check_cuda(launch_pdl(score_narrow_merge_kernel, dim3(static_cast<unsigned>(rows_all)), dim3(kThreads), 0,
-                                stream, P, part, lse2)) != APACK_OK)
-        return APACK_ECUDA;
+      const cudaError_t e =
+          max_nparts <= 32 * kHold
+              ? launch_pdl(score_narrow_merge_rows_kernel, dim3(static_cast<unsigned>((rows_all + kWarps - 1) / kWarps)),
+                           dim3(kThreads), 0, stream, P, part, lse2, static_cast<int>(rows_all))
+              : launch_pdl(score_narrow_merge_kernel, dim3(static_cast<unsigned>(rows_all)), dim3(kThreads), 0,
+                           stream, P, part, lse2);
+      if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
       count_launches(1);
     }
-    auto *final_kernel = split == 1   ? (inside ? score_narrow_final_kernel<true, 1> : score_narrow_final_kernel<false, 1>)
-                         : split == 2 ? (inside ? score_narrow_final_kernel<true, 2> : score_narrow_final_kernel<false, 2>)
-                                      : (inside ? score_narrow_final_kernel<true, 4> : score_narrow_final_kernel<false, 4>);
+    auto pick = [&](auto occ) {
+      constexpr int kOcc = decltype(occ)::value;
+      return inside       ? score_narrow_final_kernel<true, 1, kOcc>
+             : split == 1 ? score_narrow_final_kernel<false, 1, kOcc>
+             : split == 2 ? score_narrow_final_kernel<false, 2, kOcc>
+                          : score_narrow_final_kernel<false, 4, kOcc>;
+    };
+    auto *final_kernel = finals <= sms ? pick(std::integral_constant<int, 1>{}) : pick(std::integral_constant<int, 2>{});
     if (check_cuda(launch_pdl(final_kernel, dim3(finals), dim3(kFinalThreads), static_cast<size_t>(max_rows) * sizeof(float),
                               stream, P, seqs->modality, logits, part, lse2, scores)) != APACK_OK)
       return APACK_ECUDA;

@@ -141,6 +141,26 @@ def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap):
     check_scores(got, ref, strict_rel=2e-3)
 
 
+@pytest.mark.parametrize("domain", [0, 1])
+@pytest.mark.parametrize("lens,nqs,hq,hkv", [
+    ([80001], [1], 28, 4),                  # 28 rows merged in the final kernel, two of its CTAs per SM
+    ([80001], [2], 28, 4),                  # 56 rows, more than two CTAs per SM: one thread per key
+    ([40000, 0, 77], [2, 0, 0], 28, 4),     # 56 rows, two threads per key, more CTAs than SMs
+    ([19000], [4], 28, 4),                  # 112 rows, four threads per key: 149 CTAs
+    ([19800], [4], 28, 4),                  # the same with two: 155 CTAs would be four's
+    ([45001], [1], 12, 3),                  # 176 partials per row, merged in the final kernel
+    ([45001], [3], 12, 3),                  # and by one CTA per row
+])
+def test_narrow_path_final_kernel_forms(ap, lens, nqs, hq, hkv, domain):
+    """Each form of the merge and of the final kernel of the few-row path (152 SMs); the bound is the
+    one of the head layouts above."""
+    rng = np.random.default_rng(sum(lens) + 7 * hq + nqs[0])
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
+    check_scores(got, ref, strict_rel=2e-4)
+
+
 @pytest.mark.parametrize("lens,nqs,hq,hkv", SHAPES)
 def test_scores_match_oracle(ap, lens, nqs, hq, hkv):
     rng = np.random.default_rng(sum(lens) + hq)
