@@ -14,10 +14,14 @@
 //                zeroed by the pool kernel) computes c-bar, min/max of d, the min-max
 //                normalised distance and the gated score s_f of Eq. gate (blend when
 //                c-bar < tau) over the whole clip.
+//  run kernel:   in place of the pool kernel for long clips and windows 3 and 5 (below): pools a
+//                run of frames per CTA and computes the CKA of the frames inside it, so that the
+//                cka kernel is left with the frames at the runs' ends.
 // All reductions run in a fixed order: results are deterministic.  Two launches per call; the
 // CKA kernel is a programmatic dependent of the pool kernel (scheduled while the pool drains,
 // waiting for its completion before any read).
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 
 #include "internal.cuh"
@@ -294,13 +298,14 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
 
 // Per-frame windowed CKA (Eq. cka) and direct distance; the last CTA to finish also
 // runs the gate (Eq. gate) over all frames.  One CTA per frame, or with RUNS per frame at the ends
-// of runs of `run` frames (W - 1 CTAs per run), whose windows cross them.  W is the window size (odd, <= kMaxWindow);
-// windows cut by the clip's ends hold w < W rows and the missing rows are zeros that
+// of runs of `run` frames (W - 1 CTAs per run), whose windows cross them.  W is the window size (odd,
+// <= kMaxWindow); windows cut by the clip's ends hold w < W rows and the missing rows are zeros that
 // never enter a Gram entry with i or j >= w.
 // With RUNS the grid is about two CTAs per SM and its latency the call's: twice the loads in flight, and
-// the gate's inputs in registers.
+// the gate's inputs in registers.  Otherwise as many CTAs per SM as the window's rows leave registers
+// for (window 7 at 136 registers and one CTA per SM: 212 us a call of 1,200 frames, at 128 and two 190).
 template <int W, bool RUNS>
-__global__ void __launch_bounds__(kCkaThreads)
+__global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
     frame_cka_gate_kernel(const float *__restrict__ v, const float *__restrict__ a, int n_frames, int run, int64_t dim,
                           float tau, float beta, unsigned int *done, float *__restrict__ c_out,
                           float *__restrict__ d_out, float *__restrict__ s_out, float *__restrict__ dn_out,
@@ -308,7 +313,7 @@ __global__ void __launch_bounds__(kCkaThreads)
   pdl_wait_and_release();   // the pooled rows (and the zeroed counter) of the pool kernel are visible
   constexpr int kG = W * (W + 1) / 2;
   constexpr int kN = 2 * kG + 1;
-  constexpr int kHold = RUNS ? kGateHold : 1;
+  constexpr int kHold = RUNS ? kGateHold : 0;
   constexpr int kWarps = kCkaThreads / 32;
   __shared__ float red[kWarps][kN];
   __shared__ float tot[kN];
@@ -411,17 +416,19 @@ __global__ void __launch_bounds__(kCkaThreads)
   __shared__ float rmin[kWarps], rmax[kWarps];
   __shared__ double cbar_s;
   __shared__ float dmin_s, dmax_s;
-  // __ldcg: from L2, where the other CTAs' stores are
+  // from L2, where the other CTAs' stores are; one volatile load at a time keeps window 1 at 32 registers,
+  // eight CTAs per SM: a clip of 1,200 frames in one wave
   struct L2Row {
     const float *p;
     __device__ float operator[](int g) const { return __ldcg(p + g); }
   };
-  const L2Row cv{c_out}, dv{d_out};
+  using Row = std::conditional_t<RUNS, L2Row, const volatile float *>;
+  const Row cv{c_out}, dv{d_out};
   double cs = 0.0;
   float mn = INFINITY, mx = -INFINITY;
   // the first kHold frames per thread are loaded together and kept for the scores: the gate runs
   // after everything else, so its round trips are the call's (1,200 frames: 0.7 us less)
-  float ch[kHold], dh[kHold];
+  float ch[kHold ? kHold : 1], dh[kHold ? kHold : 1];
 #pragma unroll
   for (int i = 0; i < kHold; ++i) {
     const int g = threadIdx.x + i * kCkaThreads;
