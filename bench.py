@@ -566,8 +566,7 @@ def prellm_measure(ap, wl, steps, warmup, stream, dist, window=3):
     launches = ap.apack_launch_count() - n0
     ms = max_over_ranks(e0.elapsed_time(e1) / k, dist, "cuda")
     token_bytes = (F * tpf + na) * dim * 2
-    frame_bytes = 2 * F * dim * 4
-    alg = token_bytes + frame_bytes
+    alg = token_bytes + 2 * F * 4
     achieved = alg / (ms / 1e3) / 1e9
     peak, peak_kind = measured_peaks()
     prof = profiled_traffic("prellm.cu", "prellm_traffic.json")
@@ -578,12 +577,12 @@ def prellm_measure(ap, wl, steps, warmup, stream, dist, window=3):
             "config": {"workload": f"{wl.name} clip: {F} frames x {tpf} visual tokens, {na} audio tokens, d={dim}",
                        "window": window, "tau": 0.78, "beta": 0.90,
                        "l2": "inputs larger than L2 (%.2f GB of bf16 encoder tokens)" % (token_bytes / 1e9)},
-            "roofline": {"bound": "hbm", "kernel": "apack_frame_alignment call (frame_pool_kernel + "
-                                                   "frame_cka_gate_kernel)",
+            "roofline": {"bound": "hbm", "kernel": "apack_frame_alignment call (frame_run_kernel or "
+                                                   "frame_pool_kernel, + frame_cka_gate_kernel)",
                          "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": traffic, "peak_source": peak_kind,
                          "algorithmic_bytes_per_launch": alg,
-                         "note": "bf16 tokens read once + fp32 frame embeddings written once, over the whole call"}}
+                         "note": "bf16 tokens read once + two fp32 results per frame, over the whole call"}}
 
 
 def final_levels_measure(ap, pp, nsteps, mm_per_iter, steps, warmup, stream, dist):

@@ -38,9 +38,10 @@
 // blocks in pass 1, query chunks in pass 2), four B stages deep; two 256-column
 // accumulators alternate in TMEM.  Warp 0 issues TMA, warp 1 owns TMEM (and on the
 // even CTA issues the MMAs), warps 2..17 are four epilogue warpgroups; warpgroups 2b
-// and 2b + 1 read the tiles of accumulator b, 128 columns each for the CTA's 128 lanes.  Pass 1 takes each key block's masks (which keys count)
-// from a bit array that the query repack kernel writes once per call.  Operands sit in
-// 128-byte swizzled shared memory.  Persistent pairs, one CTA per SM.
+// and 2b + 1 read the tiles of accumulator b, 128 columns each for the CTA's 128 lanes.  Pass 1
+// takes each key block's masks (which keys count) from a bit array that the query repack kernel
+// writes once per call.  Operands sit in 128-byte swizzled shared memory.  Persistent pairs, one
+// CTA per SM.
 #include <cmath>
 #include <cstdio>
 
@@ -66,10 +67,12 @@ static_assert(2 * kSpan == 256 && 2 * kCols == kSpan && 4 * kCols2 == kSpan,
 // clocks a tile (the exp2 unit 1,024, TMEM loads do not overlap it) against 1,024 for the MMA, and what
 // a warp does around its tiles comes on top, since the four warps of a scheduler tend to do it at the
 // same time.  So the loops run over a warpgroup's own tiles only, the masks come in one load, and the
-// exponentials are scheduled by hand (exp_sum): pass 1 188 -> 173 us, pass 2 170 -> 162 us over
-// 135,272 keys and 7,168 rows.  Measured slower: 8 epilogue warps with 64 or 128 columns in registers
-// (209 / 178 and 258 / 185 us), all 16 warps on every tile (197 / 187), half tiles of 128 columns
-// as MMAs of their own (200 / 206: N = 128 re-reads A from shared memory).
+// exponentials are scheduled by hand (exp_sum): pass 1 188 -> 173 us, pass 2 170 -> 156 us over
+// 135,272 keys and 7,168 rows (6 us of pass 2 from its set-up running before the wait).  Measured
+// slower: 8 epilogue warps with 64 or 128 columns in registers (209 / 178 and 258 / 185 us), all 16
+// warps on every tile (197 / 187), half tiles of 128 columns as MMAs of their own (200 / 206: N =
+// 128 re-reads A from shared memory), and 2 of 16 exponentials as a degree-5 polynomial on the FMA
+// pipe (the whole call 380 -> 395 us).
 // warp 0: TMA, warp 1: TMEM (+ MMA on the even CTA), then the epilogue warps.
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr uint32_t kTmemCols = 512;    // 2 accumulators x 256 fp32 columns
