@@ -42,6 +42,7 @@
 // takes each key block's masks (which keys count) from a bit array that the query repack kernel
 // writes once per call.  Operands sit in 128-byte swizzled shared memory.  Persistent pairs, one
 // CTA per SM.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 
@@ -136,6 +137,9 @@ constexpr uint32_t kSmemBytes = kOffBars + 512;
 static_assert(sizeof(Bars) <= 512, "barrier block");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
+// Rows of a unit times partials per row up to which pass 2 merges by itself (8,780 keys, 512 rows with 19
+// each: 20.5 -> 19.3 us; 13,500 keys, 2,048 rows with 12: 27.0 -> 31.3 us).
+constexpr int kMergeInside = 16384;
 // pass 2 counters of a launch (one word per key block, 4 bits per 32 keys) in the workspace, where the
 // in-place compaction keeps its progress words later in the step
 constexpr size_t kCounterOff = 256;
@@ -713,20 +717,15 @@ __device__ float exact_nlse(const SeqPlan &sp, int g, int r, const uint16_t *__r
   return mm == -INFINITY ? INFINITY : -(mm + log2f(tot));
 }
 
-// One thread per packed query row (sequence, KV head group, rho); writes -lse2 at the row's packed index
-// (padding rows -inf, so that they add exp2(-inf) = 0).  The partials of the pair ranges that touched the
-// row group (at most 32) are taken in pair order, kBatch of them loaded together: deterministic.  Bound by
-// latency: one or two L2 round trips.  A warp per row, one partial per lane, took 25 us for 68,608 rows;
-// this takes 4.8 us.  A row with a partial marked out of range (negative sum) is recomputed exactly by
-// its warp.
+// -lse2 of a packed query row (sequence, KV head group, rho), one thread per row (padding rows -inf, so
+// that they add exp2(-inf) = 0).  The partials of the pair ranges that touched the row group (at most 32)
+// are taken in pair order, kBatch of them loaded together: deterministic.  A row with a partial marked out
+// of range (negative sum) is recomputed exactly by its warp: whole warps call this, with consecutive rows
+// (a row group is a multiple of 256 rows and never ends inside one).
 template <bool CAUSAL>
-__global__ void __launch_bounds__(kMergeThreads)
-    lse_merge_kernel(const __grid_constant__ ScorePlan plan, const float2 *__restrict__ part,
-                     const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k, int64_t k_stride,
-                     const uint8_t *__restrict__ modality, float *__restrict__ nlse2, int64_t row_begin) {
-  pdl_wait_and_release();
-  // the rows of a launch are a multiple of 256: whole CTAs, and a row group never ends inside a warp
-  const int64_t prow = row_begin + blockIdx.x * static_cast<int64_t>(kMergeThreads) + threadIdx.x;
+__device__ __forceinline__ float merged_nlse(const ScorePlan &plan, const float2 *__restrict__ part,
+                                             const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k,
+                                             int64_t k_stride, const uint8_t *__restrict__ modality, int64_t prow) {
   int s = 0;
   while (s + 1 < plan.nseq && plan.seq[s + 1].qp_base <= prow) ++s;
   const SeqPlan &sp = plan.seq[s];
@@ -772,7 +771,20 @@ __global__ void __launch_bounds__(kMergeThreads)
                                        modality);
     if (lane == l) out = x;
   }
-  nlse2[prow] = out;
+  return out;
+}
+
+// The merge as a kernel of its own.  Bound by latency: one or two L2 round trips.  A warp per row, one
+// partial per lane, took 25 us for 68,608 rows; this takes 4.8 us.
+template <bool CAUSAL>
+__global__ void __launch_bounds__(kMergeThreads)
+    lse_merge_kernel(const __grid_constant__ ScorePlan plan, const float2 *__restrict__ part,
+                     const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k, int64_t k_stride,
+                     const uint8_t *__restrict__ modality, float *__restrict__ nlse2, int64_t row_begin) {
+  pdl_wait_and_release();
+  // the rows of a launch are a multiple of 256: whole CTAs
+  const int64_t prow = row_begin + blockIdx.x * static_cast<int64_t>(kMergeThreads) + threadIdx.x;
+  nlse2[prow] = merged_nlse<CAUSAL>(plan, part, qp, k, k_stride, modality, prow);
 }
 
 // ------------------------------------------------------------------ pass 2
@@ -813,10 +825,21 @@ __device__ __forceinline__ void colsum_word_from(const uint32_t (&r)[kCols2], co
 // A unit of every group writes its keys' scores.  A unit of one group writes the group's sums to
 // gsum[g][key]; with counters the last of a key block's units then adds the groups (every warp for its
 // 32 keys), without them the final kernel does.
-template <bool CAUSAL>
+// MERGE (at most one unit per pair): there is no merge kernel; the epilogue warps merge the unit's rows
+// into shared memory while the tiles load and the first MMA runs.  A launch less in a chain of dependent
+// launches: 28/4 heads, 64 query rows, 1,298 keys 16.5 -> 15.0 us, 2,600 keys 18.2 -> 16.7 us; four
+// sequences of 600 keys 19.6 -> 17.4 us.
+struct MergeIn {
+  const float2 *part;
+  const uint16_t *qp;
+  const uint8_t *k;
+  int64_t k_stride;
+};
+
+template <bool CAUSAL, bool MERGE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     score_colsum_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
-                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2, float *gsum,
+                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2, MergeIn in, float *gsum,
                         uint32_t *counters, const uint8_t *__restrict__ modality, float *__restrict__ scores,
                         DeviceError *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -825,7 +848,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     return;
   }
   Bars *bars = reinterpret_cast<Bars *>(smem + kOffBars);
-  float *lse_s = reinterpret_cast<float *>(smem + kOffL);   // [4][256], indexed by B stage
+  float *lse_s = reinterpret_cast<float *>(smem + kOffL);   // [4][256] by B stage; MERGE: by chunk of the unit
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PairCtx pc = init_pair(smem, bars, warp);
   pdl_wait_and_release();      // the set-up runs beside the previous launch
@@ -860,10 +883,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           for (int c = 0; c < nch; ++c) {
             if (!wait_or_abort(&bars->b_empty[bi], bph ^ 1, bars, pc, err, 22)) { ok = false; break; }
             // normaliser slot bi is free once this CTA's epilogue of the chunk that used it is done
-            if (!wait_or_abort(&bars->l_empty[bi], bph ^ 1, bars, pc, err, 29)) { ok = false; break; }
+            if (!MERGE && !wait_or_abort(&bars->l_empty[bi], bph ^ 1, bars, pc, err, 29)) { ok = false; break; }
             const int64_t row0 = static_cast<int64_t>(sp.qp_base) + g * sp.rows_pad + c * kChunk;
-            mbar_arrive_expect_tx(&bars->l_full[bi], kChunk * sizeof(float));
-            bulk_load(lse_s + bi * kChunk, nlse2 + row0, kChunk * sizeof(float), &bars->l_full[bi]);
+            if (!MERGE) {
+              mbar_arrive_expect_tx(&bars->l_full[bi], kChunk * sizeof(float));
+              bulk_load(lse_s + bi * kChunk, nlse2 + row0, kChunk * sizeof(float), &bars->l_full[bi]);
+            }
             uint8_t *B = smem + kOffB + bi * kTileBytes;
             if (pc.rank == 0) mbar_arrive_expect_tx(&bars->b_full[bi], 2 * kTileBytes);
             const uint32_t bfull = lead_addr(pc, bars, &bars->b_full[bi]);
@@ -878,7 +903,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       if (!ok) {
         // this CTA's normaliser copies complete on its own barriers
-        drain_loads(bars->l_full, pend, pend_par, kBStages);
+        if (!MERGE) drain_loads(bars->l_full, pend, pend_par, kBStages);
         if (pc.rank == 0) {
           drain_loads(bars->b_full, pend, pend_par, kBStages);
           drain_loads(bars->a_full, apend, apend_par, kAStages);
@@ -937,13 +962,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (nch == 0) continue;
       // causal rows: only packed rows rho >= rho_min (tokens r >= key - q_pos) see this key
       const int rho_min = CAUSAL ? max(0, w.kp * kBlock + klane - sp.q_pos) * G : 0;
+      if (MERGE) {                                          // the pair's only unit
+        const int64_t row0 = static_cast<int64_t>(sp.qp_base) + w.g * sp.rows_pad;
+        for (int i = threadIdx.x - 64; i < plan.unit_groups * sp.rows_pad; i += 32 * kEpiWarps)
+          lse_s[i] = merged_nlse<CAUSAL>(plan, in.part, in.qp, in.k, in.k_stride, modality, row0 + i);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      }
       float mine = 0.f;                                     // the groups' sums, in group order
       for (int g = 0; ok && g < plan.unit_groups; ++g) {
         float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         // chunks alternate between the buffers; normaliser slot = chunk % kBStages, an even number
         for (int c = (own ^ tile0) & 1; c < nch; c += 2) {
-          const uint32_t t = tile0 + c, li = t % kBStages;
-          if (!wait_or_abort(&bars->l_full[li], (t / kBStages) & 1, bars, pc, err, 30)) { ok = false; break; }
+          const uint32_t t = tile0 + c, li = MERGE ? t : t % kBStages;
+          if (!MERGE && !wait_or_abort(&bars->l_full[li], (t / kBStages) & 1, bars, pc, err, 30)) { ok = false; break; }
           if (!wait_or_abort(&bars->acc_full[own], cph, bars, pc, err, 26)) { ok = false; break; }
           cph ^= 1;
           tc_fence_after();
@@ -965,7 +996,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               colsum_word_from(rr, nl, c2, first, a);
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(&bars->l_empty[li]);
+          if (!MERGE && lane == 0) mbar_arrive(&bars->l_empty[li]);
         }
         tile0 += nch;
         const float2 s01 = fadd2(a[0], a[1]), s23 = fadd2(a[2], a[3]);
@@ -1089,7 +1120,7 @@ int max_resident_pairs() {
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = kSmemBytes;
   // the kernels declare their cluster shape (__cluster_dims__), so the configuration leaves it out
-  if (cudaOccupancyMaxActiveClusters(&n, score_colsum_kernel<false>, &cfg) != cudaSuccess || n <= 0) {
+  if (cudaOccupancyMaxActiveClusters(&n, score_colsum_kernel<false, false>, &cfg) != cudaSuccess || n <= 0) {
     cudaGetLastError();
     n = device_sm_count() / 2;
   }
@@ -1138,12 +1169,9 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(score_rowstats_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kSmemBytes);
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(score_colsum_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kSmemBytes);
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(score_colsum_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kSmemBytes);
+        for (auto *f : {score_colsum_kernel<false, false>, score_colsum_kernel<true, false>,
+                        score_colsum_kernel<false, true>, score_colsum_kernel<true, true>})
+          if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         return e;
       }) != cudaSuccess)
     return APACK_ECUDA;
@@ -1241,7 +1269,13 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
-    if (qrows > 0) {
+    // Pass 2 merges the row statistics by itself where each pair has one unit, the unit's chunks fit its
+    // normaliser slots, and the rows and partials that all units read again are few (kMergeInside).
+    int64_t tiles_max = 0;
+    for (int i = 0; i < ns; ++i) tiles_max = std::max<int64_t>(tiles_max, P.unit_groups * (P.seq[i].rows_pad / kChunk));
+    const int64_t parts_max = flat > 0 ? (nb_max - 1) / (flat / pairs1) + 2 : 0;
+    const bool merge_inside = units2 <= max_pairs && tiles_max <= kBStages && tiles_max * kChunk * parts_max <= kMergeInside;
+    if (qrows > 0 && !merge_inside) {
       const cudaError_t e = launch_pdl(P.causal ? lse_merge_kernel<true> : lse_merge_kernel<false>,
                                        dim3(static_cast<unsigned>(qrows / kMergeThreads)), dim3(kMergeThreads), 0, stream,
                                        P, part, reinterpret_cast<const uint16_t *>(qp), static_cast<const uint8_t *>(k),
@@ -1253,9 +1287,11 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
     P.total_units = units2;
     if (units2 > 0) {
       const int pairs2 = units2 < max_pairs ? units2 : max_pairs;
-      const cudaError_t e = launch_pdl(P.causal ? score_colsum_kernel<true> : score_colsum_kernel<false>,
-                                       dim3(static_cast<unsigned>(2 * pairs2)), dim3(kThreads), kSmemBytes, stream, qmap,
-                                       kmap, P, nlse2, gsum, counters, seqs->modality, scores, err);
+      auto *colsum = merge_inside ? (P.causal ? score_colsum_kernel<true, true> : score_colsum_kernel<false, true>)
+                                  : (P.causal ? score_colsum_kernel<true, false> : score_colsum_kernel<false, false>);
+      const MergeIn in{part, reinterpret_cast<const uint16_t *>(qp), static_cast<const uint8_t *>(k), k_token_stride};
+      const cudaError_t e = launch_pdl(colsum, dim3(static_cast<unsigned>(2 * pairs2)), dim3(kThreads), kSmemBytes,
+                                       stream, qmap, kmap, P, nlse2, in, gsum, counters, seqs->modality, scores, err);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }

@@ -329,6 +329,34 @@ def test_scores_with_a_logit_far_above_its_run_reference(ap, domain):
     assert ref[1500] > 1e-3 and ref[1777] > 1e-3
 
 
+@pytest.mark.parametrize("domain", [0, 1])
+@pytest.mark.parametrize("lens,nqs,hq,hkv", [
+    ([600], [146], 28, 4),                  # four chunks per head group: the column pass merges
+    ([600], [147], 28, 4),                  # five: the merge kernel
+    ([8780], [64], 16, 2),                  # 19 partials per row: the column pass
+    ([900, 0, 300], [5, 0, 140], 28, 4),    # chunks of several sequences: the column pass
+    ([9000], [20], 28, 4),                  # more units than CTA pairs: the merge kernel
+])
+def test_row_statistics_merged_in_either_place(ap, lens, nqs, hq, hkv, domain):
+    """Where the partials of the row statistics meet, with and without a row marked for the exact
+    recomputation (a logit far above its run's reference, as above): equal to the oracle (tolerance of
+    test_narrow_path_head_layouts_and_row_counts) and the same bits in every call."""
+    rng = np.random.default_rng(sum(lens) + hq + domain)
+    for planted in (False, True):
+        mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=0.05 if planted else 1.5)
+        if planted:
+            key = int(cu[1]) - nqs[0] - 3
+            na = [int(x) - (mod[key] == 1) * (i == 0) for i, x in enumerate(na)]
+            nv = [int(x) + (mod[key] != 2) * (i == 0) for i, x in enumerate(nv)]
+            mod[key] = 2
+            k[key, hkv - 1] = bf16(12.0 * oracle.bf16_to_f64(q[2, hq - 1]))
+        got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+        ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
+        check_scores(got, ref, strict_rel=2e-3 if planted else 2e-4)
+        again = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+        assert got.tobytes() == again.tobytes()
+
+
 def test_scores_identical_keys_are_uniform(ap):
     mod = np.array([0] * 16 + [1, 2, 2, 2] * 300 + [0] * 8, np.uint8)
     T = mod.size
