@@ -326,13 +326,13 @@ apack_status apack_graph_destroy(apack_graph graph);
    CTAs of a sequence claim its 128-key tiles from a counter as they go, so
    the grouping of keys into partial sums, and with it the last bits of out,
    can differ from call to call (not where the caches are so short that each
-   CTA has its own tiles); the other head layouts merge in a fixed order.  ws: 256-byte aligned, apack_decode_workspace_size bytes (the size
-   depends on the device's SM count: query it on the device that runs the
-   call), zeroed by the caller once before its first use: its first 16 bytes
-   are a device error word read by apack_device_error, and its end (of the
-   ws_bytes passed: pass the same for one workspace) holds the claim
-   counters, which every call leaves at zero; caches may grow and shrink
-   from call to call.  A device-side wait that
+   CTA has its own tiles); the other head layouts merge in a fixed order.
+   ws: 256-byte aligned, apack_decode_workspace_size bytes (the size depends
+   on the device's SM count: query it on the device that runs the call),
+   zeroed by the caller once before its first use: its first 16 bytes are a
+   device error word read by apack_device_error, and bytes 256..511 hold the
+   claim counters, which every call leaves at zero.  Batch, caches and ws_bytes
+   may change from call to call on one workspace.  A device-side wait that
    runs out records APACK_ETIMEOUT there.  Two kernel launches per 64
    sequences; no allocation, no synchronisation. */
 apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seqlens_h, int32_t num_q_heads,

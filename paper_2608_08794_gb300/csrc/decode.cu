@@ -344,8 +344,8 @@ cudaError_t launch_chunk(int grid, cudaStream_t stream, const DecPlan &P, const 
 // One CTA of WARPS warps per (sequence, query head): merge the sequence's chunks.  Warp w folds chunks
 // w, w + WARPS, w + 2 WARPS, ... in that order (lane: features [4 lane, 4 lane + 4)); the warps
 // then merge in warp order.  A sequence with no cached token gets zeros.  The CTA of query
-// head 0 also zeroes the sequence's stage-claim counter for the next call (the chunk kernel,
-// the counter's only user, is complete here).
+// head 0 also zeroes the sequence's stage-claim counters for the next launch (the chunk kernel,
+// their only user, is complete here).
 template <int WARPS>
 __global__ void __launch_bounds__(32 * WARPS)
     decode_combine_kernel(const __grid_constant__ DecPlan plan, const float *__restrict__ opart,
@@ -435,6 +435,26 @@ apack_status decode_validate(int32_t num_seqs, const int32_t *cu_seqlens_h, int3
 
 size_t up256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
+// Workspace: device error word; the claim counters of a launch, one per sequence (a call of one sequence:
+// one per head share, at most four); chunk partials o [chunks][Hq][128], then (max, sum) [chunks][Hq].
+// The counters lie in front of everything whose size follows the call, so that they are at the same bytes,
+// and zero, whatever batch, caches and ws_bytes an earlier call on the workspace had; the launches of a
+// call share them (a launch's combine zeroes them before the next launch's chunk kernel starts on them).
+constexpr size_t kClaimsOff = 256;
+constexpr size_t kPartsOff = kClaimsOff + kSeqsPerLaunch * sizeof(unsigned int);
+static_assert(kPartsOff % 256 == 0, "float4 partials");
+
+size_t decode_bytes(int64_t chunks, int32_t hq) {
+  return kPartsOff + up256(static_cast<size_t>(chunks) * hq * 128 * sizeof(float)) +
+         up256(static_cast<size_t>(chunks) * hq * sizeof(float2));
+}
+
+int64_t decode_chunks(int32_t num_seqs, const int32_t *cu_seqlens_h, int chunk) {
+  int64_t chunks = 0;
+  for (int b = 0; b < num_seqs; ++b) chunks += (static_cast<int64_t>(cu_seqlens_h[b + 1]) - cu_seqlens_h[b] + chunk - 1) / chunk;
+  return chunks;
+}
+
 }  // namespace
 
 }  // namespace apack
@@ -449,14 +469,7 @@ apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seq
   int64_t total = 0;
   const apack_status st = decode_validate(num_seqs, cu_seqlens_h, num_q_heads, num_kv_heads, &total);
   if (st != APACK_OK) return st;
-  const int chunk = decode_chunk_keys(num_seqs, cu_seqlens_h);
-  int64_t chunks = 0;
-  for (int b = 0; b < num_seqs; ++b) chunks += (cu_seqlens_h[b + 1] - cu_seqlens_h[b] + chunk - 1) / chunk;
-  // device error word, chunk partials o [chunks][Hq][128] and (max, sum) [chunks][Hq], one
-  // stage-claim counter per sequence
-  *bytes = 256 + up256(static_cast<size_t>(chunks) * num_q_heads * 128 * sizeof(float)) +
-           up256(static_cast<size_t>(chunks) * num_q_heads * sizeof(float2)) +
-           up256(static_cast<size_t>(num_seqs) * sizeof(unsigned int));
+  *bytes = decode_bytes(decode_chunks(num_seqs, cu_seqlens_h, decode_chunk_keys(num_seqs, cu_seqlens_h)), num_q_heads);
   return APACK_OK;
 }
 
@@ -474,20 +487,15 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
       (reinterpret_cast<uintptr_t>(ws) & 255) || (kv_token_stride & 15) ||
       kv_token_stride < static_cast<int64_t>(num_kv_heads) * 256)
     return APACK_EINVAL;
-  size_t need = 0;
-  apack_decode_workspace_size(num_seqs, cu_seqlens_h, num_q_heads, num_kv_heads, &need);
-  if (ws_bytes < need) return APACK_EWORKSPACE;
   const int chunk = decode_chunk_keys(num_seqs, cu_seqlens_h);
-  int64_t chunks_all = 0;
-  for (int b = 0; b < num_seqs; ++b) chunks_all += (cu_seqlens_h[b + 1] - cu_seqlens_h[b] + chunk - 1) / chunk;
+  const int64_t chunks_all = decode_chunks(num_seqs, cu_seqlens_h, chunk);
+  if (ws_bytes < decode_bytes(chunks_all, num_q_heads)) return APACK_EWORKSPACE;
+  uint8_t *wsb = static_cast<uint8_t *>(ws);
   DeviceError *err = static_cast<DeviceError *>(ws);
-  float *opart = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + 256);
-  float2 *mlpart = reinterpret_cast<float2 *>(static_cast<uint8_t *>(ws) + 256 +
+  unsigned int *claims = reinterpret_cast<unsigned int *>(wsb + kClaimsOff);
+  float *opart = reinterpret_cast<float *>(wsb + kPartsOff);
+  float2 *mlpart = reinterpret_cast<float2 *>(wsb + kPartsOff +
                                               up256(static_cast<size_t>(chunks_all) * num_q_heads * 128 * sizeof(float)));
-  // the claim counters lie at the end of the workspace that the caller passed, not after this call's
-  // partials: they stay where they are, and zero, when the caches grow or shrink between calls
-  const size_t claims_off = (ws_bytes - up256(static_cast<size_t>(num_seqs) * sizeof(unsigned int))) & ~static_cast<size_t>(255);
-  unsigned int *claims = reinterpret_cast<unsigned int *>(static_cast<uint8_t *>(ws) + claims_off);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t *q16 = static_cast<const uint16_t *>(q);
   const bool tc = decode_tc_applies(num_q_heads, num_kv_heads) && total > 0;
@@ -536,7 +544,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     const uint16_t *qs = q16 + static_cast<int64_t>(s0) * num_q_heads * 128;
     if (chunks > 0) {
       if (tc) {
-        if (check_cuda(launch_decode_tc(chunks << P.split_log, s, kmap, vmap, P, qs, op, mp, claims + s0, err)) != APACK_OK)
+        if (check_cuda(launch_decode_tc(chunks << P.split_log, s, kmap, vmap, P, qs, op, mp, claims, err)) != APACK_OK)
           return APACK_ECUDA;
       } else {
         auto *launch = P.group > 4 ? launch_chunk<8> : P.group > 2 ? launch_chunk<4> : P.group > 1 ? launch_chunk<2>
@@ -552,7 +560,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     const bool few = max_chunks <= kDecCombineFew * kDecCombineBatch;
     if (check_cuda(launch_pdl(few ? decode_combine_kernel<kDecCombineFew> : decode_combine_kernel<kDecCombineMany>,
                               dim3(ns * num_q_heads), dim3(32 * (few ? kDecCombineFew : kDecCombineMany)), 0, s, P, op, mp,
-                              out + static_cast<int64_t>(s0) * num_q_heads * 128, claims + s0)) != APACK_OK)
+                              out + static_cast<int64_t>(s0) * num_q_heads * 128, claims)) != APACK_OK)
       return APACK_ECUDA;
     count_launches(1);
     chunk_base += chunks;
