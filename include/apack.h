@@ -332,7 +332,8 @@ apack_status apack_graph_destroy(apack_graph graph);
    zeroed by the caller once before its first use: its first 16 bytes are a
    device error word read by apack_device_error, and bytes 256..511 hold the
    claim counters, which every call leaves at zero.  Batch, caches and ws_bytes
-   may change from call to call on one workspace.  A device-side wait that
+   may change from call to call on one workspace; the size for the longest
+   caches serves every shorter one of as many sequences.  A device-side wait that
    runs out records APACK_ETIMEOUT there.  Two kernel launches per 64
    sequences; no allocation, no synchronisation. */
 apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seqlens_h, int32_t num_q_heads,

@@ -400,6 +400,8 @@ bool decode_tc_applies(int32_t hq, int32_t hkv) { return (hkv == 2 || hkv == 4) 
 // CTA per SM over the whole batch, and then as many as bring every launch (kSeqsPerLaunch sequences) down
 // to one CTA per SM, within 1/16: a last chunk per sequence that starts a second round of CTAs costs as
 // much as the first (48 caches of 100 to 3,000 tokens, 28/4 heads: 55.2 -> 38.6 us).
+constexpr int64_t kMaxChunkKeys = 1 << 20;
+
 int decode_chunk_keys(int32_t num_seqs, const int32_t *cu_seqlens_h) {
   const int64_t ctas = std::max(1, device_sm_count());
   const int64_t total = num_seqs > 0 ? cu_seqlens_h[num_seqs] : 0;
@@ -418,7 +420,7 @@ int decode_chunk_keys(int32_t num_seqs, const int32_t *cu_seqlens_h) {
       c = whole(c + std::max<int64_t>(1, c / 16));
     }
   }
-  return static_cast<int>(std::min<int64_t>(c, 1 << 20));
+  return static_cast<int>(std::min<int64_t>(c, kMaxChunkKeys));
 }
 
 apack_status decode_validate(int32_t num_seqs, const int32_t *cu_seqlens_h, int32_t hq, int32_t hkv,
@@ -455,6 +457,17 @@ int64_t decode_chunks(int32_t num_seqs, const int32_t *cu_seqlens_h, int chunk) 
   return chunks;
 }
 
+// Chunks of this batch or of one with shorter caches, at most: decode_chunk_keys leaves a launch one CTA per
+// SM, or one chunk per sequence (of kMaxChunkKeys keys).  Fewer keys can mean more chunks (152 SMs: 19,456
+// keys 152 chunks, 19,457 keys 77), so a workspace for the longest caches needs the bound, not their count.
+int64_t decode_chunks_bound(int32_t num_seqs, const int32_t *cu_seqlens_h) {
+  int64_t bound = 0;
+  for (int s0 = 0; s0 < num_seqs; s0 += kSeqsPerLaunch)
+    bound += std::max<int64_t>(device_sm_count(), decode_chunks(std::min(num_seqs - s0, kSeqsPerLaunch),
+                                                                cu_seqlens_h + s0, static_cast<int>(kMaxChunkKeys)));
+  return bound;
+}
+
 }  // namespace
 
 }  // namespace apack
@@ -469,7 +482,7 @@ apack_status apack_decode_workspace_size(int32_t num_seqs, const int32_t *cu_seq
   int64_t total = 0;
   const apack_status st = decode_validate(num_seqs, cu_seqlens_h, num_q_heads, num_kv_heads, &total);
   if (st != APACK_OK) return st;
-  *bytes = decode_bytes(decode_chunks(num_seqs, cu_seqlens_h, decode_chunk_keys(num_seqs, cu_seqlens_h)), num_q_heads);
+  *bytes = decode_bytes(decode_chunks_bound(num_seqs, cu_seqlens_h), num_q_heads);
   return APACK_OK;
 }
 

@@ -91,6 +91,22 @@ def test_keep_counts_match_oracle_rule(ap):
         ap.apack_keep_counts(s, np.full((B, 2), 1.5, np.float32))
 
 
+@pytest.mark.parametrize("hq,hkv", [(28, 4), (8, 8)])
+def test_decode_workspace_for_the_longest_caches_serves_shorter_ones(ap, hq, hkv):
+    """The size never grows when caches get shorter, although their chunks can get more."""
+    rng = np.random.default_rng(hq)
+
+    def size(lens):
+        return ap.apack_decode_workspace_size(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), hq, hkv)
+
+    assert size([700] * 20 + [2500] * 44) <= size([2500] * 64)
+    assert size([19456]) <= size([19457]) and size([18944]) <= size([18945])
+    for _ in range(200):
+        lens = rng.integers(0, rng.choice([300, 5000, 40000]), rng.choice([1, 3, 16, 48, 64, 70, 130]))
+        assert size((lens * rng.random(len(lens))).astype(int)) <= size(lens)
+        assert size((lens * rng.random()).astype(int)) <= size(lens)
+
+
 def test_calls_reject_bad_arguments_before_the_device(ap):
     import torch  # noqa: F401  (CPU tensors only: pointers are never dereferenced)
     s = make_seqs(ap)
