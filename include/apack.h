@@ -245,7 +245,10 @@ apack_status apack_score_static(const apack_seqs *seqs, const void *q, const voi
    n_audio >= n_frames >= 1, window odd in 1..7 (the paper uses 3, tau = 0.78,
    beta = 0.90).  Outputs (device, fp32): c_out [F], s_out [F], dnorm_out [F]
    (nullable), cbar_out [1] (nullable).  fp32 accumulation, fixed reduction
-   order (deterministic).  ws: 256-byte aligned, apack_frame_alignment_workspace_size. */
+   order (deterministic).  ws: 256-byte aligned, apack_frame_alignment_workspace_size
+   bytes, not zeroed: every call writes the device error word in its first 16
+   bytes (apack_device_error).  A device-side wait that runs out records
+   APACK_ETIMEOUT there, and every output of the call is NaN. */
 apack_status apack_frame_alignment_workspace_size(int32_t n_frames, int64_t dim, size_t *bytes);
 apack_status apack_frame_alignment(const void *visual, const void *audio, int32_t n_frames,
                                    int32_t tokens_per_frame, int32_t n_audio, int64_t dim, int32_t window,

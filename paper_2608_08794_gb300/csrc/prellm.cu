@@ -146,17 +146,35 @@ __device__ __forceinline__ float cka_of(const float *tot) {
   return den > 0.f ? dot / den : 0.f;
 }
 
+// A bounded wait that also gives up when another thread of the CTA has; one that runs out sets the flag.
+__device__ __forceinline__ bool run_wait(uint64_t *bar, uint32_t parity, volatile unsigned int *gave_up) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  for (;;) {
+    for (int i = 0; i < 32; ++i)
+      if (mbar_try_wait(bar, parity)) return true;
+    if (*gave_up) return false;
+    if (globaltimer_ns() - t0 > kWaitLimitNs) {
+      *gave_up = 1;
+      return false;
+    }
+  }
+}
+
+// status[run]: 1 when a wait of the run's CTA gave up (its sums are then not to be used), else 0.
 template <int W>
 __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
     frame_run_kernel(const __grid_constant__ RunShape sh, const uint8_t *__restrict__ visual,
                      const uint8_t *__restrict__ audio, float *__restrict__ v_out, float *__restrict__ a_out,
-                     float *__restrict__ c_out, float *__restrict__ d_out, unsigned int *done) {
+                     float *__restrict__ c_out, float *__restrict__ d_out, unsigned int *done,
+                     unsigned int *__restrict__ status) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the CKA kernel may be scheduled
   constexpr int kH = W / 2, kG = W * (W + 1) / 2, kN = 2 * kG + 1;
   extern __shared__ __align__(128) uint8_t ring[];
   __shared__ __align__(8) uint64_t full[kRunStages], empty[kRunStages];
   __shared__ float red[run_threads<W>() / 32][kN];
   __shared__ float tot[kN];
+  __shared__ volatile unsigned int gave_up;
   const int nthr = blockDim.x - 32, nwarps = nthr / 32;               // consumers
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t row = sh.dim * 2;                                     // bytes of a token row, a multiple of 16
@@ -167,6 +185,7 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], nwarps);
     }
+    gave_up = 0;
     fence_mbar_init();
     if (blockIdx.x == 0) *done = 0u;                                  // CTA counter of the CKA kernel
   }
@@ -178,7 +197,7 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
       auto stream = [&](const uint8_t *src, int64_t rows) -> bool {
         for (int64_t r = 0; r < rows; r += stage_rows, ++n) {
           const int slot = n % kRunStages;
-          if (n >= kRunStages && !mbar_wait(&empty[slot], (n / kRunStages - 1) & 1u, kWaitLimitNs)) return false;
+          if (n >= kRunStages && !run_wait(&empty[slot], (n / kRunStages - 1) & 1u, &gave_up)) return false;
           const uint32_t bytes = static_cast<uint32_t>(min(static_cast<int64_t>(stage_rows), rows - r) * row);
           mbar_arrive_expect_tx(&full[slot], bytes);
           bulk_load(ring + slot * kRunStage, src + r * row, bytes, &full[slot]);
@@ -191,9 +210,10 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
         const int64_t j0 = audio_begin(f, sh.n_audio, sh.n_frames), j1 = audio_begin(f + 1, sh.n_audio, sh.n_frames);
         if (ok) ok = stream(audio + j0 * row, j1 - j0);
       }
-      if (!ok)   // copies in flight land before the CTA exits
-        for (uint32_t i = n > kRunStages ? n - kRunStages : 0; i < n; ++i)
-          mbar_wait(&full[i % kRunStages], (i / kRunStages) & 1u, kWaitLimitNs / 4);
+      // no copy lands after the CTA has left, whoever gave up: the last of every slot is awaited here (the
+      // ones before were consumed)
+      for (uint32_t i = n > kRunStages ? n - kRunStages : 0; i < n; ++i)
+        if (!mbar_wait(&full[i % kRunStages], (i / kRunStages) & 1u, kWaitLimitNs)) gave_up = 1;
     }
     return;
   }
@@ -206,10 +226,11 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
     for (int i = 0; i < 8; ++i) acc[i] = 0.f;
     for (int64_t r = 0; r < rows; r += stage_rows, ++n) {
       const int slot = n % kRunStages;
-      if (ok && !__all_sync(0xffffffffu, mbar_wait(&full[slot], (n / kRunStages) & 1u, kWaitLimitNs))) ok = false;
+      if (ok && !__all_sync(0xffffffffu, run_wait(&full[slot], (n / kRunStages) & 1u, &gave_up))) ok = false;
+      if (!ok) continue;                          // no barrier is touched after a wait that failed
       const int cnt = static_cast<int>(min(static_cast<int64_t>(stage_rows), rows - r));
       const uint8_t *p = ring + slot * kRunStage + tid * 16;
-      if (mine && ok)
+      if (mine)
 #pragma unroll 4
         for (int i = 0; i < cnt; ++i) add_bf16x8(*reinterpret_cast<const uint4 *>(p + i * row), acc);
       __syncwarp();
@@ -287,13 +308,14 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
       }
       __syncwarp();
       if (lane == 0) {
-        // a wait that gave up shows as NaN
-        c_out[f - kH] = ok ? cka_of<W>(tot) : NAN;
+        c_out[f - kH] = cka_of<W>(tot);
         d_out[f - kH] = sqrtf(tot[2 * kG]);
       }
     }
     asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");   // red is free again
   }
+  asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");     // every consumer's last wait is over
+  if (tid == 0) status[blockIdx.x] = gave_up;
 }
 
 // Per-frame windowed CKA (Eq. cka) and direct distance; the last CTA to finish also
@@ -302,14 +324,17 @@ __global__ void __launch_bounds__(run_threads<W>() + 32, 1)
 // <= kMaxWindow); windows cut by the clip's ends hold w < W rows and the missing rows are zeros that
 // never enter a Gram entry with i or j >= w.
 // With RUNS the grid is about two CTAs per SM and its latency the call's: twice the loads in flight, and
-// the gate's inputs in registers.  Otherwise as many CTAs per SM as the window's rows leave registers
+// the gate's inputs in registers (two CTAs per SM stated: left open, the compiler takes 64 registers for
+// window 3 in place of 96, and the call of 1,200 frames 158 us in place of 155.5).  Otherwise as many CTAs per SM as the window's rows leave registers
 // for (window 7 at 136 registers and one CTA per SM: 212 us a call of 1,200 frames, at 128 and two 190).
+// The last CTA also writes the device error word.  If a run gave up a wait, every output is NaN: the
+// gate's mean and range need all frames.
 template <int W, bool RUNS>
-__global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
+__global__ void __launch_bounds__(kCkaThreads, W == 7 || RUNS ? 2 : 0)
     frame_cka_gate_kernel(const float *__restrict__ v, const float *__restrict__ a, int n_frames, int run, int64_t dim,
                           float tau, float beta, unsigned int *done, float *__restrict__ c_out,
                           float *__restrict__ d_out, float *__restrict__ s_out, float *__restrict__ dn_out,
-                          float *__restrict__ cbar_out) {
+                          float *__restrict__ cbar_out, const unsigned int *status, DeviceError *err) {
   pdl_wait_and_release();   // the pooled rows (and the zeroed counter) of the pool kernel are visible
   constexpr int kG = W * (W + 1) / 2;
   constexpr int kN = 2 * kG + 1;
@@ -317,10 +342,12 @@ __global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
   constexpr int kWarps = kCkaThreads / 32;
   __shared__ float red[kWarps][kN];
   __shared__ float tot[kN];
-  __shared__ bool last;
+  __shared__ bool last, gave_up;
   int f = blockIdx.x;
+  unsigned int bad = 0;                                     // thread 0: this CTA's run gave up a wait
   if (RUNS) {
     constexpr int kPer = W > 1 ? W - 1 : 1;                 // 2 (W / 2) frames per run
+    if (threadIdx.x == 0) bad = __ldcg(status + f / kPer);
     const int f0 = f / kPer * run, f1 = min(n_frames, f0 + run), i = f % kPer;
     // a last run shorter than W - 1 frames: the CTAs past it take its last frame again
     f = i < W / 2 ? min(f0 + i, f1 - 1) : max(f1 - kPer + i, f0);
@@ -406,7 +433,10 @@ __global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
     c_out[f] = cka_of<W>(tot);
     d_out[f] = sqrtf(tot[2 * kG]);
     __threadfence();
-    last = atomicAdd(done, 1u) == gridDim.x - 1;
+    // with RUNS the count's upper half counts the CTAs whose run gave up (a grid is a few CTAs per SM)
+    const unsigned int add = 1u + (bad << 16), now = atomicAdd(done, add) + add;
+    last = (RUNS ? now & 0xffffu : now) == gridDim.x;
+    gave_up = RUNS && now >> 16;
   }
   __syncthreads();
   if (!last) return;
@@ -461,6 +491,8 @@ __global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    err->code = gave_up ? APACK_ETIMEOUT : APACK_OK;
+    err->where = gave_up ? 71 : 0;
     double t = 0.0;
     float lo_d = INFINITY, hi_d = -INFINITY;
     for (int wp = 0; wp < kWarps; ++wp) {
@@ -468,7 +500,7 @@ __global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
       lo_d = fminf(lo_d, rmin[wp]);
       hi_d = fmaxf(hi_d, rmax[wp]);
     }
-    cbar_s = t / n_frames;
+    cbar_s = gave_up ? static_cast<double>(NAN) : t / n_frames;
     dmin_s = lo_d;
     dmax_s = hi_d;
     if (cbar_out) *cbar_out = static_cast<float>(cbar_s);
@@ -477,7 +509,8 @@ __global__ void __launch_bounds__(kCkaThreads, W == 7 ? 2 : 0)
   const bool blend = cbar_s < static_cast<double>(tau);
   const float span = dmax_s - dmin_s;
   auto gate = [&](int g, float cg, float dg) {
-    const float dn = span > 0.f ? (dg - dmin_s) / span : 0.f;
+    float dn = span > 0.f ? (dg - dmin_s) / span : 0.f;
+    if (RUNS && gave_up) c_out[g] = cg = dn = NAN;
     if (dn_out) dn_out[g] = dn;
     s_out[g] = blend ? (1.f - beta) * cg + beta * (1.f - dn) : cg;
   };
@@ -499,7 +532,7 @@ extern "C" {
 
 apack_status apack_frame_alignment_workspace_size(int32_t n_frames, int64_t dim, size_t *bytes) {
   if (!bytes || n_frames < 1 || dim < 8) return APACK_EINVAL;
-  // error word, v [F][dim], a [F][dim], c [F], d [F], scratch
+  // device error word and CTA counter, v [F][dim], a [F][dim], d [F], status [runs <= F], unused
   *bytes = 256 + 2 * up(static_cast<size_t>(n_frames) * dim * sizeof(float)) +
            2 * up(static_cast<size_t>(n_frames) * sizeof(float)) + 256;
   return APACK_OK;
@@ -520,10 +553,12 @@ apack_status apack_frame_alignment(const void *visual, const void *audio, int32_
   apack_frame_alignment_workspace_size(n_frames, dim, &need);
   if (ws_bytes < need) return APACK_EWORKSPACE;
   uint8_t *w = static_cast<uint8_t *>(ws);
-  unsigned int *done = reinterpret_cast<unsigned int *>(w);
+  DeviceError *err = reinterpret_cast<DeviceError *>(w);
+  unsigned int *done = reinterpret_cast<unsigned int *>(w + 64);
   float *vbuf = reinterpret_cast<float *>(w + 256);
   float *abuf = reinterpret_cast<float *>(w + 256 + up(static_cast<size_t>(n_frames) * dim * sizeof(float)));
   float *dbuf = reinterpret_cast<float *>(w + 256 + 2 * up(static_cast<size_t>(n_frames) * dim * sizeof(float)));
+  unsigned int *status = reinterpret_cast<unsigned int *>(reinterpret_cast<uint8_t *>(dbuf) + up(static_cast<size_t>(n_frames) * sizeof(float)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t vecs = dim / 8;
   const int pthreads = static_cast<int>(std::min<int64_t>(kPoolMaxThreads, (vecs + 31) / 32 * 32));
@@ -552,7 +587,7 @@ apack_status apack_frame_alignment(const void *visual, const void *audio, int32_
         }) != cudaSuccess)
       return APACK_ECUDA;
     kernel<<<runs, pthreads + 32, smem, s>>>(sh, static_cast<const uint8_t *>(visual), static_cast<const uint8_t *>(audio),
-                                             vbuf, abuf, c_out, dbuf, done);
+                                             vbuf, abuf, c_out, dbuf, done, status);
     cka_run = run;
     cka_grid = runs * (window - 1);
   } else {
@@ -568,7 +603,7 @@ apack_status apack_frame_alignment(const void *visual, const void *audio, int32_
               : window == 5 ? (cka_run ? frame_cka_gate_kernel<5, true> : frame_cka_gate_kernel<5, false>)
                             : frame_cka_gate_kernel<7, false>;
   const cudaError_t e = launch_pdl(cka, dim3(cka_grid), dim3(kCkaThreads), 0, s, vbuf, abuf, n_frames, cka_run, dim, tau,
-                                   beta, done, c_out, dbuf, s_out, dnorm_out, cbar_out);
+                                   beta, done, c_out, dbuf, s_out, dnorm_out, cbar_out, status, err);
   count_launches(1);
   if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
   return APACK_OK;

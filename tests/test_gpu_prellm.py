@@ -38,6 +38,7 @@ def run(ap, vis, aud, F, tpf, dim, window, tau, beta):
     ap.apack_frame_alignment(v_d, a_d, F, tpf, aud.shape[0], dim, c, s, ws, window=window, tau=tau, beta=beta,
                              dnorm_out=dn, cbar_out=cb)
     torch.cuda.synchronize()
+    assert ap.apack_device_error(ws) == ap.APACK_OK      # written by every call
     return c.cpu().numpy(), s.cpu().numpy(), dn.cpu().numpy(), float(cb.item())
 
 
