@@ -109,7 +109,10 @@ typedef struct apack_plane {
 } apack_plane;
 
 /* Bytes of device workspace the calls below need for this batch (256-byte
-   aligned start required).  Depends on B, the query rows and head counts. */
+   aligned start required).  Depends on B, the query rows and head counts.
+   Bytes 0..15 are the device error word, bytes 256..1023 belong to the
+   in-place compaction of apack_compact; everything else is scratch that the
+   scoring writes before it reads. */
 apack_status apack_workspace_size(const apack_seqs *seqs, size_t *bytes);
 
 /* Keep counts of Eq. inner, ceil((1-P)|S|), from keep ratios r = 1-P.
@@ -135,7 +138,7 @@ apack_status apack_keep_counts(const apack_seqs *seqs, const float *keep_ratio_h
    k: bf16 keys of the pruning layer, token t at k + t*k_token_stride, laid
       out [Hkv][D] within the row; k_token_stride a multiple of 16 bytes.
    scores: fp32 [T].  Computed in fp32 from bf16 products on the tensor
-   cores; deterministic (fixed reduction order, no atomics).  q and k must be
+   cores; deterministic (fixed reduction order).  q and k must be
    device memory (they are read by TMA; host memory gives APACK_EINVAL). */
 apack_status apack_score(const apack_seqs *seqs, const void *q, const void *k, int64_t k_token_stride,
                          float *scores, void *ws, size_t ws_bytes, void *stream);

@@ -140,10 +140,11 @@ static_assert(kSmemBytes <= 232448, "shared memory budget");
 // Rows of a unit times partials per row up to which pass 2 merges by itself (8,780 keys, 512 rows with 19
 // each: 20.5 -> 19.3 us; 13,500 keys, 2,048 rows with 12: 27.0 -> 31.3 us).
 constexpr int kMergeInside = 16384;
-// pass 2 counters of a launch (one word per key block, 4 bits per 32 keys) in the workspace, where the
-// in-place compaction keeps its progress words later in the step
-constexpr size_t kCounterOff = 256;
-constexpr int kMaxCounted = 192;               // key blocks
+// pass 2 counters of a launch (one word per key block, 4 bits per 32 keys) in the workspace, between the
+// error word and the words of the in-place compaction, which may run beside a scoring on the workspace.
+// A counted call has at most as many blocks as half the GPU's CTA pairs (38 with 152 SMs).
+constexpr size_t kCounterOff = sizeof(DeviceError);
+constexpr int kMaxCounted = (256 - static_cast<int>(kCounterOff)) / 4;   // key blocks
 constexpr int kMaxCountedGroups = 15;          // what 4 bits count
 
 __device__ __forceinline__ bool is_mm(uint8_t m) { return m == APACK_MOD_AUDIO || m == APACK_MOD_VISUAL; }

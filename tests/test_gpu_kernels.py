@@ -195,6 +195,26 @@ def test_column_pass_modes(ap, lens, nqs, hq, hkv, domain):
     assert got.tobytes() == again.tobytes()
 
 
+def test_scoring_leaves_the_compactions_words_alone(ap):
+    """Bytes 256..1023 of a workspace are the in-place compaction's (it may run on another stream): a call
+    whose last unit of a key block adds the head groups keeps its counters elsewhere, and clears them
+    for itself whatever an earlier call left."""
+    lens, nqs, hq, hkv = [4000, 255], [40, 40], 28, 4
+    rng = np.random.default_rng(5)
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
+    mod_d, q_d, k_d = dev(mod), dev(q), dev(k)
+    seqs = ap.Seqs(cu, cuq, na, nv, mod_d, hq, hkv)
+    ws = aligned_ws(ap, seqs)
+    ws[16:] = 0x5A                                          # all but the error word
+    scores = torch.full((int(cu[-1]),), float("nan"), dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        ap.apack_score(seqs, q_d, k_d, hkv * D * 2, scores, ws)
+        torch.cuda.synchronize()
+        assert ap.apack_device_error(ws) == ap.APACK_OK
+        assert bool((ws[256:1024] == 0x5A).all())
+        check_scores(scores.cpu().numpy(), oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv), strict_rel=2e-4)
+
+
 # ------------------------------------------------------------------------------ causal-row domain
 
 CAUSAL_SHAPES = [
