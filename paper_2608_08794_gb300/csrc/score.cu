@@ -11,8 +11,7 @@
 //     contiguous ranges, one per CTA pair; a pair writes one partial (m, sum) per
 //     row for each row group its range touches.
 //  merge: per packed query row, the partials combine in pair order into a log2-domain
-//     normaliser lse2 = log2 sum_j 2^(x_j log2(e)/sqrt(D)), stored negated (a row whose
-//     logits overflowed its run's reference is recomputed there exactly).
+//     normaliser lse2 = log2 sum_j 2^(x_j log2(e)/sqrt(D)), stored negated.
 //  pass 2 (column sums): D[key][row] = K . Q^T with keys in TMEM lanes; each
 //     thread owns one key and sums 2^(x c - lse2[row]) over the rows of one KV
 //     head group; the Hkv group sums are added in a fixed order and scaled by
@@ -123,6 +122,7 @@ struct __align__(8) Bars {
   uint64_t comb_full[2], comb_empty[2];           // column ranges 1.. -> range 0 hand-off
   uint32_t tmem_base;
   volatile int32_t abort;
+  volatile int32_t marked;                        // pass 1: the CTA wrote a partial with a sum out of range
 };
 
 // Shared memory: [A x2][B x4][-lse2 x4 (pass 2)][combine 2 x (kEpiWG - 1) x 128 float2][Bars].
@@ -280,6 +280,7 @@ __device__ PairCtx init_pair(uint8_t *smem, Bars *bars, int warp) {
     }
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
+    bars->marked = 0;
     fence_mbar_init();
   }
   pc.lead_bars = map_shared_rank(bars, 0);
@@ -377,7 +378,7 @@ __device__ __forceinline__ Run next_run(const ScorePlan &p, int x, int x_end, in
 // every mask.  The reference is the first counted block's maximum and stays fixed for the
 // run: no block's sums feed back into the next block's arithmetic.  A block whose sum leaves
 // the safe range (a logit more than about 2^99 above the reference, or an overflow) only sets
-// `bad`; such a row's normaliser is recomputed exactly by the merge kernel.  Four independent
+// `bad`; such a partial is recomputed exactly at the CTA's end (repair_marked).  Four independent
 // partial sums keep the add chains short.
 constexpr float kSumLimit = 6.338253e29f;   // 2^99
 
@@ -444,10 +445,81 @@ __device__ __forceinline__ void online_block(uint32_t (&r)[64], uint32_t mask0, 
   sum += t;
 }
 
+// The (maximum, sum) in log2 units of one query row qr over the keys of blocks [b0, b1) of a sequence,
+// computed by a warp without the tensor cores.  kg: the head group's keys of the sequence; words: its key
+// masks; keys past `see` do not count.  One key per lane: dot products in fp32 from the bf16 values, an
+// online sum with exact rescaling, the lanes combined in a fixed order.
+__device__ __forceinline__ float2 exact_part(const uint4 *__restrict__ qr, const uint8_t *__restrict__ kg, int64_t k_stride,
+                                             const uint32_t *__restrict__ words, int b0, int b1, int see) {
+  const int lane = threadIdx.x & 31;
+  float m = -INFINITY, sum = 0.f;
+  for (int w = b0 * (kBlock / 32); w < b1 * (kBlock / 32); ++w) {
+    const int key = w * 32 + lane;
+    if (!((__ldg(words + w) >> lane) & 1u) || key > see) continue;
+    const uint4 *kr = reinterpret_cast<const uint4 *>(kg + key * k_stride);
+    float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 4
+    for (int d = 0; d < 16; ++d) {
+      const uint4 q8 = __ldg(qr + d), k8 = __ldg(kr + d);
+      const uint32_t qw[4] = {q8.x, q8.y, q8.z, q8.w}, kw[4] = {k8.x, k8.y, k8.z, k8.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        a[e] = ffma2(make_float2(__uint_as_float(qw[e] << 16), __uint_as_float(qw[e] & 0xFFFF0000u)),
+                     make_float2(__uint_as_float(kw[e] << 16), __uint_as_float(kw[e] & 0xFFFF0000u)), a[e]);
+    }
+    const float2 t = fadd2(fadd2(a[0], a[1]), fadd2(a[2], a[3]));
+    const float y = (t.x + t.y) * kScale2;                // not from the tensor cores
+    if (y > m) {
+      sum = (m == -INFINITY ? 0.f : sum * exp2f(m - y)) + 1.f;
+      m = y;
+    } else {
+      sum += exp2f(y - m);
+    }
+  }
+  __syncwarp();
+  float mm = m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+  float tot = m != -INFINITY ? sum * exp2f(m - mm) : sum;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  return make_float2(mm, tot);
+}
+
+// Computes the partials that a CTA marked (a negative sum) again, its warps a row each.  The work stays in
+// the row's run, so it is spread over the GPU like the runs, and the merge finds every partial in range.
+// With every row marked, against whole rows recomputed in the merge by a warp per row and by a warp per 32
+// rows: 135,272 keys, 256 x 28 rows, 67 ms against 640 and 963; 8,780 keys, 64 x 16 rows, 0.16 ms against 29
+// and 232.  As a call at the end of each run it took the tile loop's registers (370 -> 390 us without a mark).
+template <bool CAUSAL>
+__device__ __noinline__ void repair_marked(const ScorePlan &plan, int pair, int row_half,
+                                           const uint32_t *__restrict__ mask_words, const uint4 *__restrict__ qp,
+                                           const uint8_t *__restrict__ k, int64_t k_stride, float2 *part) {
+  const int G = plan.group;
+  const int x_end = range_start(pair + 1, plan.pairs, plan.flat_total);
+  for (int x = range_start(pair, plan.pairs, plan.flat_total); x < x_end;) {
+    const Run w = next_run(plan, x, x_end, pair);
+    const SeqPlan &sp = plan.seq[w.s];
+    x = w.x1;
+    for (int row = row_half + (threadIdx.x >> 5); row < row_half + kRows; row += kThreads / 32) {
+      const int rho = w.qp * kChunk + row;                    // linear row of the head group
+      if (rho >= G * sp.n_q) break;
+      const int r = rho / G, j = rho - r * G;
+      float2 *p = part + (static_cast<size_t>(w.slot) * plan.total_qrows + sp.q_off + r) * plan.hq + w.g * G + j;
+      if (!(p->y < 0.f)) continue;
+      const float2 v = exact_part(qp + (sp.qp_base + static_cast<int64_t>(w.g) * sp.rows_pad + rho) * 16,
+                                  k + sp.t0 * k_stride + w.g * 256, k_stride, mask_words + sp.blk0 * 8, w.b0, w.b1,
+                                  CAUSAL ? sp.q_pos + r : sp.len);
+      if ((threadIdx.x & 31) == 0) *p = v;
+    }
+  }
+}
+
 template <bool CAUSAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     score_rowstats_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                           const __grid_constant__ ScorePlan plan, const uint32_t *__restrict__ mask_words,
+                          const uint4 *__restrict__ qp, const uint8_t *__restrict__ k, int64_t k_stride,
                           float2 *__restrict__ part, DeviceError *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   if (!smem_aligned(smem)) {   // the same in both CTAs of the pair: both leave here
@@ -592,7 +664,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (!ok) break;
       // the column ranges of each row combine in a fixed order (range 0 writes the pair's
       // partial of the row group; the merge combines the pairs' partials in pair order).  A
-      // sum out of range travels as a negative sum: the merge then recomputes the row.
+      // sum out of range travels as a negative sum: the CTA recomputes the partial at its end.
       if (bad) sum = -1.f;
       float2 *cb = comb + (xph & 1) * (kEpiWG - 1) * kRows;
       const int trow = quad * 32 + lane;
@@ -628,12 +700,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const int r = rho / G, j = rho - r * G;
           part[(static_cast<size_t>(w.slot) * plan.total_qrows + sp.q_off + r) * plan.hq + w.g * G + j] =
               make_float2(mm, tot);
+          if (flagged) bars->marked = 1;
         }
       }
       ++xph;
     }
   }
   finish_pair(bars, pc, warp, warp == 1 && lane == 0 && pc.rank == 0);
+  // the epilogue's stores are visible to the whole CTA after finish_pair's barriers
+  if (bars->marked && !bars->abort) repair_marked<CAUSAL>(plan, pair, row_half, mask_words, qp, k, k_stride, part);
 }
 
 // ------------------------------------------------------------------ repack
@@ -682,51 +757,10 @@ __global__ void q_pack_kernel(const __grid_constant__ ScorePlan plan, const uint
 }
 
 // ------------------------------------------------------------------ merge
-// Negated log2 normaliser of one query row (token r of the span, packed row qr) of KV head group g,
-// computed by a warp without the tensor cores: the lanes take every 32nd key of the sequence, dot it
-// with the row in fp32 from the bf16 values, keep an online (max, sum of exp2) with exact rescaling, and
-// combine in a fixed order.  Slow, and only taken for inputs whose logits span more than about 99
-// binary orders of magnitude (a partial marked by a negative sum).
-template <bool CAUSAL>
-__device__ float exact_nlse(const SeqPlan &sp, int g, int r, const uint16_t *__restrict__ qr,
-                                         const uint8_t *__restrict__ k, int64_t k_stride,
-                                         const uint8_t *__restrict__ modality) {
-  const int see = sp.q_pos + r;                         // causal rows: keys up to the row's position
-  float m = -INFINITY, sum = 0.f;
-  for (int key = sp.t0 + (threadIdx.x & 31); key < sp.t0 + sp.len; key += 32) {
-    if (CAUSAL ? key - sp.t0 > see : !is_mm(modality[key])) continue;
-    const uint16_t *kr = reinterpret_cast<const uint16_t *>(k + key * k_stride) + g * 128;
-    float dot = 0.f;
-#pragma unroll 8
-    for (int d = 0; d < 128; ++d)
-      dot = fmaf(__uint_as_float(static_cast<uint32_t>(qr[d]) << 16), __uint_as_float(static_cast<uint32_t>(kr[d]) << 16),
-                 dot);
-    const float y = dot * kScale2;                      // not from the tensor cores
-    if (y > m) {
-      sum = (m == -INFINITY ? 0.f : sum * exp2f(m - y)) + 1.f;
-      m = y;
-    } else {
-      sum += exp2f(y - m);
-    }
-  }
-  float mm = m;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-  float tot = (m != -INFINITY) ? sum * exp2f(m - mm) : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-  return mm == -INFINITY ? INFINITY : -(mm + log2f(tot));
-}
-
 // -lse2 of a packed query row (sequence, KV head group, rho), one thread per row (padding rows -inf, so
 // that they add exp2(-inf) = 0).  The partials of the pair ranges that touched the row group (at most 32)
-// are taken in pair order, kBatch of them loaded together: deterministic.  A row with a partial marked out
-// of range (negative sum) is recomputed exactly by its warp: whole warps call this, with consecutive rows
-// (a row group is a multiple of 256 rows and never ends inside one).
-template <bool CAUSAL>
-__device__ __forceinline__ float merged_nlse(const ScorePlan &plan, const float2 *__restrict__ part,
-                                             const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k,
-                                             int64_t k_stride, const uint8_t *__restrict__ modality, int64_t prow) {
+// are taken in pair order, kBatch of them loaded together: deterministic.
+__device__ __forceinline__ float merged_nlse(const ScorePlan &plan, const float2 *__restrict__ part, int64_t prow) {
   int s = 0;
   while (s + 1 < plan.nseq && plan.seq[s + 1].qp_base <= prow) ++s;
   const SeqPlan &sp = plan.seq[s];
@@ -741,7 +775,6 @@ __device__ __forceinline__ float merged_nlse(const ScorePlan &plan, const float2
                                  pair_of(x0, plan.pairs, plan.flat_total) + 1
                            : 0;
   float out = -INFINITY;
-  bool exact = false;
   if (real) {
     const float2 *p = part + static_cast<size_t>(sp.q_off + r) * plan.hq + g * G + j;
     const size_t stride = static_cast<size_t>(plan.total_qrows) * plan.hq;
@@ -758,34 +791,24 @@ __device__ __forceinline__ float merged_nlse(const ScorePlan &plan, const float2
       if (m != -INFINITY) tot *= exp2f(m - mn);
 #pragma unroll
       for (int i = 0; i < kBatch; ++i) {
-        exact |= v[i].y < 0.f;
         if (v[i].x != -INFINITY) tot += v[i].y * exp2f(v[i].x - mn);
       }
       m = mn;
     }
     out = m == -INFINITY ? INFINITY : -(m + log2f(tot));   // no key at all (S empty): nothing is scored
   }
-  const int lane = threadIdx.x & 31;
-  for (uint32_t todo = __ballot_sync(0xffffffffu, exact); todo; todo &= todo - 1) {
-    const int l = __ffs(todo) - 1;
-    const float x = exact_nlse<CAUSAL>(sp, g, __shfl_sync(0xffffffffu, r, l), qp + (prow - lane + l) * 128, k, k_stride,
-                                       modality);
-    if (lane == l) out = x;
-  }
   return out;
 }
 
 // The merge as a kernel of its own.  Bound by latency: one or two L2 round trips.  A warp per row, one
 // partial per lane, took 25 us for 68,608 rows; this takes 4.8 us.
-template <bool CAUSAL>
 __global__ void __launch_bounds__(kMergeThreads)
     lse_merge_kernel(const __grid_constant__ ScorePlan plan, const float2 *__restrict__ part,
-                     const uint16_t *__restrict__ qp, const uint8_t *__restrict__ k, int64_t k_stride,
-                     const uint8_t *__restrict__ modality, float *__restrict__ nlse2, int64_t row_begin) {
+                     float *__restrict__ nlse2, int64_t row_begin) {
   pdl_wait_and_release();
   // the rows of a launch are a multiple of 256: whole CTAs
   const int64_t prow = row_begin + blockIdx.x * static_cast<int64_t>(kMergeThreads) + threadIdx.x;
-  nlse2[prow] = merged_nlse<CAUSAL>(plan, part, qp, k, k_stride, modality, prow);
+  nlse2[prow] = merged_nlse(plan, part, prow);
 }
 
 // ------------------------------------------------------------------ pass 2
@@ -830,17 +853,10 @@ __device__ __forceinline__ void colsum_word_from(const uint32_t (&r)[kCols2], co
 // into shared memory while the tiles load and the first MMA runs.  A launch less in a chain of dependent
 // launches: 28/4 heads, 64 query rows, 1,298 keys 16.5 -> 15.0 us, 2,600 keys 18.2 -> 16.7 us; four
 // sequences of 600 keys 19.6 -> 17.4 us.
-struct MergeIn {
-  const float2 *part;
-  const uint16_t *qp;
-  const uint8_t *k;
-  int64_t k_stride;
-};
-
 template <bool CAUSAL, bool MERGE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     score_colsum_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
-                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2, MergeIn in, float *gsum,
+                        const __grid_constant__ ScorePlan plan, const float *__restrict__ nlse2, const float2 *__restrict__ part, float *gsum,
                         uint32_t *counters, const uint8_t *__restrict__ modality, float *__restrict__ scores,
                         DeviceError *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -966,7 +982,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (MERGE) {                                          // the pair's only unit
         const int64_t row0 = static_cast<int64_t>(sp.qp_base) + w.g * sp.rows_pad;
         for (int i = threadIdx.x - 64; i < plan.unit_groups * sp.rows_pad; i += 32 * kEpiWarps)
-          lse_s[i] = merged_nlse<CAUSAL>(plan, in.part, in.qp, in.k, in.k_stride, modality, row0 + i);
+          lse_s[i] = merged_nlse(plan, part, row0 + i);
         asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
       }
       float mine = 0.f;                                     // the groups' sums, in group order
@@ -1266,7 +1282,8 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
     if (flat > 0) {
       const cudaError_t e = launch_pdl(P.causal ? score_rowstats_kernel<true> : score_rowstats_kernel<false>,
                                        dim3(static_cast<unsigned>(2 * pairs1)), dim3(kThreads), kSmemBytes, stream, qmap,
-                                       kmap, P, mask_words, part, err);
+                                       kmap, P, mask_words, reinterpret_cast<const uint4 *>(qp),
+                                       static_cast<const uint8_t *>(k), k_token_stride, part, err);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
@@ -1277,10 +1294,8 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
     const int64_t parts_max = flat > 0 ? (nb_max - 1) / (flat / pairs1) + 2 : 0;
     const bool merge_inside = units2 <= max_pairs && tiles_max <= kBStages && tiles_max * kChunk * parts_max <= kMergeInside;
     if (qrows > 0 && !merge_inside) {
-      const cudaError_t e = launch_pdl(P.causal ? lse_merge_kernel<true> : lse_merge_kernel<false>,
-                                       dim3(static_cast<unsigned>(qrows / kMergeThreads)), dim3(kMergeThreads), 0, stream,
-                                       P, part, reinterpret_cast<const uint16_t *>(qp), static_cast<const uint8_t *>(k),
-                                       k_token_stride, seqs->modality, nlse2, qp_base);
+      const cudaError_t e = launch_pdl(lse_merge_kernel, dim3(static_cast<unsigned>(qrows / kMergeThreads)),
+                                       dim3(kMergeThreads), 0, stream, P, part, nlse2, qp_base);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }
@@ -1290,9 +1305,8 @@ apack_status run_score(const apack_seqs *seqs, const void *q, const void *k, int
       const int pairs2 = units2 < max_pairs ? units2 : max_pairs;
       auto *colsum = merge_inside ? (P.causal ? score_colsum_kernel<true, true> : score_colsum_kernel<false, true>)
                                   : (P.causal ? score_colsum_kernel<true, false> : score_colsum_kernel<false, false>);
-      const MergeIn in{part, reinterpret_cast<const uint16_t *>(qp), static_cast<const uint8_t *>(k), k_token_stride};
       const cudaError_t e = launch_pdl(colsum, dim3(static_cast<unsigned>(2 * pairs2)), dim3(kThreads), kSmemBytes,
-                                       stream, qmap, kmap, P, nlse2, in, gsum, counters, seqs->modality, scores, err);
+                                       stream, qmap, kmap, P, nlse2, part, gsum, counters, seqs->modality, scores, err);
       count_launches(1);
       if (check_cuda(e) != APACK_OK) return APACK_ECUDA;
     }

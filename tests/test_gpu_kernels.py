@@ -331,8 +331,8 @@ def test_scores_large_logits_and_sequence_without_S(ap):
 def test_scores_with_a_logit_far_above_its_run_reference(ap, domain):
     """A late key aligned with one query row gives that row a logit about 190 binary orders of
     magnitude above the maximum of the first key block: the row's online sum would overflow
-    its run's fixed reference, so the pass-1 partial is marked and the merge recomputes the
-    row's normaliser exactly.  Scores must still match the oracle on every token of S."""
+    its run's fixed reference, so the pass-1 partial is marked and computed again
+    exactly.  Scores must still match the oracle on every token of S."""
     rng = np.random.default_rng(99 + domain)
     mod, cu, cuq, k, q, na, nv = random_batch(rng, [2000], [5], 28, 4, scale_k=0.05)
     h, r = 9, 2                                    # query head 9 (KV head 1), query row 2
@@ -347,6 +347,45 @@ def test_scores_with_a_logit_far_above_its_run_reference(ap, domain):
     ref = oracle.relevance_scores(q, k, cu, cuq, mod, 28, 4, softmax_domain=domain)
     check_scores(got, ref)
     assert ref[1500] > 1e-3 and ref[1777] > 1e-3
+
+
+@pytest.mark.parametrize("domain", [0, 1])
+@pytest.mark.parametrize("lens,nqs,hq,hkv", [
+    ([8780], [64], 16, 2),                  # the column pass merges the partials
+    ([7000], [10], 8, 1),                   # the merge kernel; 80 rows of 256
+    ([3000, 0, 700], [30, 0, 40], 28, 4),
+])
+def test_scores_with_every_row_out_of_its_reference_range(ap, lens, nqs, hq, hkv, domain):
+    """Logits that spread over hundreds of binary orders mark partials of most rows.  Scores equal the
+    oracle (a logit of up to 500 binary orders in fp32 is off by at most 128 2^-24 of the sum of its terms'
+    magnitudes, 4e-3; 2e-3 holds with the terms' random signs), and the marked partials cost no
+    more than the work they are: the call within 100 times that of the same shape without any (4 to
+    9 times here; 8,000 times where one warp took 32 whole rows)."""
+    rng = np.random.default_rng(sum(lens) + hq + domain)
+    times = []
+    for scale in (1.0, 7.0):
+        mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=scale, scale_q=scale)
+        mod_d, q_d, k_d = dev(mod), dev(q), dev(k)
+        seqs = ap.Seqs(cu, cuq, na, nv, mod_d, hq, hkv, softmax_domain=domain)
+        ws = aligned_ws(ap, seqs)
+        scores = torch.full((int(cu[-1]),), float("nan"), dtype=torch.float32, device="cuda")
+        best = float("inf")
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ap.apack_score(seqs, q_d, k_d, hkv * D * 2, scores, ws)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+        assert ap.apack_device_error(ws) == ap.APACK_OK
+        got = scores.cpu().numpy().astype(np.float64)
+        ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
+        # terms below 2^-126 are 0 in fp32, so a score is off by up to that: 2e-3 of it from 2^-117 on
+        small = ref < 2.0 ** -116
+        assert (got[small] <= 2.0 ** -115).all()
+        check_scores(np.where(small, 0, got), np.where(small, 0, ref))
+    assert times[1] < 100 * times[0], times
 
 
 @pytest.mark.parametrize("domain", [0, 1])
