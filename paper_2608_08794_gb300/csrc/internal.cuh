@@ -71,7 +71,7 @@ int device_sm_count();
 void count_launches(uint64_t n);
 apack_status check_cuda(cudaError_t e);
 
-// Programmatic dependent launch.  The scoring kernels (both paths), selection, the out-of-place gather,
+// Programmatic dependent launch.  The scoring kernels (but the CUDA-core logits), selection, the out-of-place gather,
 // the decode kernels and the frame CKA are launched with programmatic stream serialization: a kernel may
 // be scheduled while its predecessor on the stream drains, and it waits (griddepcontrol.wait, before any
 // global access of what that launch may write) until the predecessor has completed and its memory is

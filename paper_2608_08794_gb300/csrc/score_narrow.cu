@@ -364,8 +364,11 @@ cudaError_t launch_logits(int grid, size_t smem, cudaStream_t stream, const Narr
                                 160 * 1024);
   });
   if (e != cudaSuccess) return e;
-  return launch_pdl(score_narrow_logits_kernel<RG>, dim3(grid), dim3(kThreads), smem, stream, P, q, k, k_stride,
-                    modality, logits, part);
+  // Not a programmatic dependent: up to six of its CTAs fit an SM, and those that start while the previous
+  // launch drains pile up on the SMs it leaves first (8 sequences of 5,000 keys, 16/16 heads, four query
+  // rows, 160 CTAs: 474 us a call among others as a dependent, 214 us so).
+  score_narrow_logits_kernel<RG><<<grid, kThreads, smem, stream>>>(P, q, k, k_stride, modality, logits, part);
+  return cudaGetLastError();
 }
 
 }  // namespace

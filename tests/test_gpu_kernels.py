@@ -141,6 +141,35 @@ def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap):
     check_scores(got, ref, strict_rel=2e-3)
 
 
+def test_narrow_path_general_logits_spread_over_the_sms(ap):
+    """The CUDA-core logits kernel of a call must not pile its CTAs up on the SMs that the call before
+    leaves first: a call among others takes no longer than one that starts on an idle GPU (2.4 times as
+    long when it started beside the other's last kernel; 30 % for the measurement)."""
+    lens, nqs, hq, hkv = [5000] * 8, [4] * 8, 16, 16       # 160 CTAs of 256 keys
+    rng = np.random.default_rng(3)
+    mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv)
+    mod_d, q_d, k_d = dev(mod), dev(q), dev(k)
+    seqs = ap.Seqs(cu, cuq, na, nv, mod_d, hq, hkv)
+    ws = aligned_ws(ap, seqs)
+    scores = torch.empty(int(cu[-1]), dtype=torch.float32, device="cuda")
+
+    def best(calls):
+        times = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(calls):
+                ap.apack_score(seqs, q_d, k_d, hkv * D * 2, scores, ws)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) / calls)
+        return min(times)
+
+    alone, among = best(1), best(12)
+    assert among < 1.3 * alone, (among, alone)
+
+
 @pytest.mark.parametrize("domain", [0, 1])
 @pytest.mark.parametrize("lens,nqs,hq,hkv", [
     ([80001], [1], 28, 4),                  # 28 rows merged in the final kernel, two of its CTAs per SM
