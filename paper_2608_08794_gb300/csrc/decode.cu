@@ -399,7 +399,9 @@ bool decode_tc_applies(int32_t hq, int32_t hkv) { return (hkv == 2 || hkv == 4) 
 // Keys per chunk, whole 128-key tiles (a multiple of every stage size of both chunk kernels): about one
 // CTA per SM over the whole batch, and then as many as bring every launch (kSeqsPerLaunch sequences) down
 // to one CTA per SM, within 1/16: a last chunk per sequence that starts a second round of CTAs costs as
-// much as the first (48 caches of 100 to 3,000 tokens, 28/4 heads: 55.2 -> 38.6 us).
+// much as the first (48 caches of 100 to 3,000 tokens, 28/4 heads: 55.2 -> 38.6 us).  Not where the second
+// round would hold short chunks only and a chunk's time is its arithmetic (64/8 heads, one cache of 60,000
+// tokens before 63 of 300: 134.9 -> 151.6 us).
 constexpr int64_t kMaxChunkKeys = 1 << 20;
 
 int decode_chunk_keys(int32_t num_seqs, const int32_t *cu_seqlens_h) {
