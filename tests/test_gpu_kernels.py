@@ -61,14 +61,22 @@ def random_batch(rng, lens, nqs, hq, hkv, p_other=0.05, scale_k=1.0, scale_q=1.0
     return mod, cu, cuq, k, q, na, nv
 
 
-def gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=0, q_start=None):
+def forms_of_152_sms():
+    """Which kernels a shape takes depends on the SM count; the shapes below are those of 152 SMs."""
+    return torch.cuda.get_device_properties(0).multi_processor_count == 152
+
+
+def gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=0, q_start=None, launches=None):
     mod_d = dev(mod)
     seqs = ap.Seqs(cu, cuq, na, nv, mod_d, hq, hkv, softmax_domain=softmax_domain, q_start=q_start)
     ws = aligned_ws(ap, seqs)
     T = int(cu[-1])
     scores = torch.full((max(T, 1),), float("nan"), dtype=torch.float32, device="cuda")
     q_d = dev(q) if q.size else torch.zeros(16, dtype=torch.int16, device="cuda")
+    before = ap.apack_launch_count()
     ap.apack_score(seqs, q_d, dev(k), hkv * D * 2, scores, ws)
+    if launches is not None and forms_of_152_sms():
+        assert ap.apack_launch_count() - before == launches, "another form than the one named"
     torch.cuda.synchronize()
     assert ap.apack_device_error(ws) == ap.APACK_OK
     return scores[:T].cpu().numpy()
@@ -129,11 +137,12 @@ def test_narrow_path_head_layouts_and_row_counts(ap, hq, hkv, nq, domain):
     check_scores(got, ref, strict_rel=2e-4)
 
 
-def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap):
-    """The general logits kernel writes one partial per 256 keys.  A batch of more than 256 keys per
+@pytest.mark.parametrize("hq,hkv", [(28, 4), (12, 3)])
+def test_narrow_path_partials_of_a_large_batch_do_not_overlap(ap, hq, hkv):
+    """The general logits kernel (three KV heads) writes one partial per 256 keys.  A batch of more than 256 keys per
     SM (38,912 tokens on 152 SMs) is one where a sequence has more of those than the tensor-core
     kernel's chunks: every sequence's partials need their own place all the same."""
-    lens, nqs, hq, hkv = [21000, 17011, 9003], [2, 3, 1], 28, 4
+    lens, nqs = [21000, 17011, 9003], [2, 3, 1]
     rng = np.random.default_rng(77)
     mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
     got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv)
@@ -171,21 +180,22 @@ def test_narrow_path_general_logits_spread_over_the_sms(ap):
 
 
 @pytest.mark.parametrize("domain", [0, 1])
-@pytest.mark.parametrize("lens,nqs,hq,hkv", [
-    ([80001], [1], 28, 4),                  # 28 rows merged in the final kernel, two of its CTAs per SM
-    ([80001], [2], 28, 4),                  # 56 rows, more than two CTAs per SM: one thread per key
-    ([40000, 0, 77], [2, 0, 0], 28, 4),     # 56 rows, two threads per key, more CTAs than SMs
-    ([19000], [4], 28, 4),                  # 112 rows, four threads per key: 149 CTAs
-    ([19800], [4], 28, 4),                  # the same with two: 155 CTAs would be four's
-    ([45001], [1], 12, 3),                  # 176 partials per row, merged in the final kernel
-    ([45001], [3], 12, 3),                  # and by one CTA per row
+@pytest.mark.parametrize("lens,nqs,hq,hkv,launches", [
+    ([80001], [1], 28, 4, 2),               # 28 rows merged in the final kernel, two of its CTAs per SM
+    ([80001], [2], 28, 4, 3),               # 56 rows, more than two CTAs per SM: one thread per key
+    ([40000, 0, 77], [2, 0, 0], 28, 4, 3),  # 56 rows, two threads per key, more CTAs than SMs
+    ([19000], [4], 28, 4, 3),               # 112 rows, four threads per key: 149 CTAs
+    ([19800], [4], 28, 4, 3),               # the same with two: 155 CTAs would be four's
+    ([45001], [1], 12, 3, 2),               # 176 partials per row, merged in the final kernel
+    ([45001], [3], 12, 3, 3),               # and by one CTA per row
 ])
-def test_narrow_path_final_kernel_forms(ap, lens, nqs, hq, hkv, domain):
-    """Each form of the merge and of the final kernel of the few-row path (152 SMs); the bound is the
-    one of the head layouts above."""
+def test_narrow_path_final_kernel_forms(ap, lens, nqs, hq, hkv, launches, domain):
+    """Each form of the merge and of the final kernel of the few-row path (152 SMs; a merge kernel shows as
+    a launch); the bound is the one of the head layouts above."""
     rng = np.random.default_rng(sum(lens) + 7 * hq + nqs[0])
     mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
-    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain,
+                         launches=launches)
     ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
     check_scores(got, ref, strict_rel=2e-4)
 
@@ -204,20 +214,22 @@ def test_scores_match_oracle(ap, lens, nqs, hq, hkv):
 
 
 @pytest.mark.parametrize("domain", [0, 1])
-@pytest.mark.parametrize("lens,nqs,hq,hkv", [
-    ([19000], [20], 28, 4),                 # units of every head group: the unit writes the scores
-    ([19000, 257], [20, 0], 28, 4),         # a sequence without query rows: the final kernel
-    ([9000], [20], 28, 4),                  # more units than CTA pairs: the final kernel
-    ([4000, 0, 255], [40, 0, 40], 28, 4),   # one unit per pair: the last of a key block adds the groups
-    ([1000], [40], 16, 16),                 # as many, but more groups than the counters count
-    ([5000], [40], 8, 1),                   # one head group
+@pytest.mark.parametrize("lens,nqs,hq,hkv,launches", [
+    # repack, pass 1, pass 2, and the merge and final kernels where the form has them
+    ([19000], [20], 28, 4, 4),              # units of every head group: the unit writes the scores (merge)
+    ([19000, 257], [20, 0], 28, 4, 5),      # a sequence without query rows: the final kernel (both)
+    ([9000], [20], 28, 4, 5),               # more units than CTA pairs: the final kernel (both)
+    ([4000, 0, 255], [40, 0, 40], 28, 4, 3),   # one unit per pair: the last of a key block adds the groups
+    ([1000], [40], 16, 16, 4),              # as many, but more groups than the counters count (final)
+    ([5000], [40], 8, 1, 3),                # one head group
 ])
-def test_column_pass_modes(ap, lens, nqs, hq, hkv, domain):
+def test_column_pass_modes(ap, lens, nqs, hq, hkv, launches, domain):
     """The ways in which the head groups' sums meet, equal to the oracle (tolerance of
     test_narrow_path_head_layouts_and_row_counts) and the same bits in every call."""
     rng = np.random.default_rng(sum(lens) + hq + domain)
     mod, cu, cuq, k, q, na, nv = random_batch(rng, lens, nqs, hq, hkv, scale_k=1.5)
-    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+    got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain,
+                         launches=launches)
     ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
     check_scores(got, ref, strict_rel=2e-4)
     again = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
@@ -418,14 +430,14 @@ def test_scores_with_every_row_out_of_its_reference_range(ap, lens, nqs, hq, hkv
 
 
 @pytest.mark.parametrize("domain", [0, 1])
-@pytest.mark.parametrize("lens,nqs,hq,hkv", [
-    ([600], [146], 28, 4),                  # four chunks per head group: the column pass merges
-    ([600], [147], 28, 4),                  # five: the merge kernel
-    ([8780], [64], 16, 2),                  # 19 partials per row: the column pass
-    ([900, 0, 300], [5, 0, 140], 28, 4),    # chunks of several sequences: the column pass
-    ([9000], [20], 28, 4),                  # more units than CTA pairs: the merge kernel
+@pytest.mark.parametrize("lens,nqs,hq,hkv,launches", [
+    ([600], [146], 28, 4, 3),               # four chunks per head group: the column pass merges
+    ([600], [147], 28, 4, 4),               # five: the merge kernel
+    ([8780], [64], 16, 2, 3),               # 19 partials per row: the column pass
+    ([900, 0, 300], [5, 0, 140], 28, 4, 3),    # chunks of several sequences: the column pass
+    ([9000], [20], 28, 4, 5),               # more units than CTA pairs: the merge kernel (and the final one)
 ])
-def test_row_statistics_merged_in_either_place(ap, lens, nqs, hq, hkv, domain):
+def test_row_statistics_merged_in_either_place(ap, lens, nqs, hq, hkv, launches, domain):
     """Where the partials of the row statistics meet, with and without a row marked for the exact
     recomputation (a logit far above its run's reference, as above): equal to the oracle (tolerance of
     test_narrow_path_head_layouts_and_row_counts) and the same bits in every call."""
@@ -438,7 +450,8 @@ def test_row_statistics_merged_in_either_place(ap, lens, nqs, hq, hkv, domain):
             nv = [int(x) + (mod[key] != 2) * (i == 0) for i, x in enumerate(nv)]
             mod[key] = 2
             k[key, hkv - 1] = bf16(12.0 * oracle.bf16_to_f64(q[2, hq - 1]))
-        got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)
+        got = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain,
+                         launches=launches)
         ref = oracle.relevance_scores(q, k, cu, cuq, mod, hq, hkv, softmax_domain=domain)
         check_scores(got, ref, strict_rel=2e-3 if planted else 2e-4)
         again = gpu_scores(ap, mod, cu, cuq, k, q, na, nv, hq, hkv, softmax_domain=domain)

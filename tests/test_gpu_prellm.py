@@ -96,6 +96,29 @@ def test_frame_alignment_runs_of_frames(ap, F, tpf, na, dim, window, tau):
     assert c.tobytes() == again[0].tobytes() and s.tobytes() == again[1].tobytes()
 
 
+@pytest.mark.parametrize("per_sm,extra,tpf,dim,window,runs", [
+    (3, 1, 25, 2048, 3, True),        # runs of 4 frames, 409,600 bytes of visual tokens each
+    (3, 1, 24, 2048, 3, True),        # 393,216 bytes, the least of a run
+    (3, 1, 23, 2048, 3, False),       # fewer: one CTA per frame
+    (2, 1, 50, 2048, 3, True),        # runs of 3 frames, the window
+    (2, 0, 50, 2048, 3, False),       # of 2
+    (4, 1, 25, 3584, 5, True),        # the widest rows of window 5
+    (4, 1, 25, 3592, 5, False),
+    (4, 1, 25, 2048, 7, False),       # window 7 has no runs
+])
+def test_frame_alignment_takes_runs_where_its_rule_says(ap, per_sm, extra, tpf, dim, window, runs):
+    """The forms do not differ in launches: runs leave a zero status word each, behind the distances."""
+    F = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    v = torch.zeros(F * tpf, dim, dtype=torch.bfloat16, device="cuda")
+    out = torch.empty(2, F, dtype=torch.float32, device="cuda")
+    ws = torch.full((ap.apack_frame_alignment_workspace_size(F, dim),), 0xA5, dtype=torch.uint8, device="cuda")
+    ap.apack_frame_alignment(v, v, F, tpf, F, dim, out[0], out[1], ws, window=window)
+    torch.cuda.synchronize()
+    up = lambda x: (x + 255) // 256 * 256
+    status = ws[256 + 2 * up(4 * F * dim) + up(4 * F):][:4]
+    assert bool((status == 0).all()) == runs
+
+
 def test_frame_alignment_two_and_a_half_minute_clip(ap):
     # 300 frames of 100 visual tokens, 25 audio tokens per second at 2 fps, 7B hidden size
     F, tpf, na, dim = 300, 100, 3750, 3584
