@@ -78,10 +78,9 @@ WsLayout workspace_layout(const apack_seqs *s) {
   const int64_t NQ = s->cu_qlens_h[s->num_seqs];
   const int64_t T = s->cu_seqlens_h[s->num_seqs];
   const int G = s->num_q_heads / s->num_kv_heads;
-  int64_t chunks = 0, qp_rows = 0;
+  int64_t qp_rows = 0;
   for (int b = 0; b < s->num_seqs; ++b) {
     const int64_t rows = static_cast<int64_t>(G) * (s->cu_qlens_h[b + 1] - s->cu_qlens_h[b]);
-    chunks += static_cast<int64_t>(s->num_kv_heads) * ((rows + 127) / 128);
     qp_rows += static_cast<int64_t>(s->num_kv_heads) * ((rows + 255) / 256) * 256;
   }
   auto up = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
@@ -99,7 +98,6 @@ WsLayout workspace_layout(const apack_seqs *s) {
   L.part_off = 1024;
   const size_t part_bytes = static_cast<size_t>(kMaxSplits) * NQ * s->num_q_heads * sizeof(float2);
   L.lse_off = up(L.part_off + part_bytes);
-  L.lse_chunks = chunks;
   L.qp_off = up(L.lse_off + static_cast<size_t>(qp_rows) * sizeof(float));
   L.qp_rows = qp_rows;
   L.gsum_off = up(L.qp_off + static_cast<size_t>(qp_rows) * 256);

@@ -527,7 +527,7 @@ apack_status apack_decode_attention(int32_t num_seqs, const int32_t *cu_seqlens_
     P.hkv = num_kv_heads;
     P.group = num_q_heads / num_kv_heads;
     P.chunk = chunk;                    // whole 128-key tiles
-    P.scale2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(APACK_HEAD_DIM)));
+    P.scale2 = kScale2;
     int chunks = 0, max_chunks = 0;
     for (int i = 0; i < ns; ++i) {
       DecSeq &d = P.seq[i];

@@ -28,7 +28,9 @@ constexpr float kScale2 = 0.12751743082459868f;
 // the fp32 accumulators of tcgen05.mma are truncated, which leaves a dot product of 128 bf16 pairs
 // 1.1e-7 of its magnitude too small on average (measured against 64 bits), and the softmax turns that
 // into a bias of the large logits.  Scores of the 5-minute sequence with three query tokens: 2.4e-7
-// off in the 2-norm with kScale2, 1.4e-7 with this.
+// off in the 2-norm with kScale2, 1.4e-7 with this.  It corrects a mean only.  Decode attention keeps
+// kScale2: its error has other terms (P as pairs of bf16, sums of V), 2.6e-6 with either over 135,000
+// tokens, 2.9e-6 and 2.4e-6 with keys of twice the spread.
 constexpr float kScale2Tc = 0.12751744687557220f;
 
 // Device error word at offset 0 of the workspace.
@@ -57,11 +59,10 @@ struct WsLayout {
   size_t mask_off;    // uint32 [key blocks of the batch][8]: which keys of a block count (pass 1)
   // few query rows per head group (narrow path, used instead of the four above):
   bool narrow;
-  size_t nlog_off;    // float [sum over sequences of Hq n_q len]: log2-domain logits
+  size_t nlog_off;    // float [sum over sequences of Hq n_q rows of len, rounded up to 64]: dot products
   size_t npart_off;   // float2 [sum of Hq n_q ctas]: per-CTA row (max, sum of exp2)
   size_t nlse_off;    // float [sum of Hq n_q]: log2 normalisers
   size_t total;
-  int64_t lse_chunks;
   int64_t qp_rows;
 };
 

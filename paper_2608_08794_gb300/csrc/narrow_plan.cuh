@@ -26,8 +26,6 @@ struct NSeq {
 
 struct NarrowPlan {
   int32_t nseq;
-  int32_t total_units;
-  int32_t total_units8;
   int32_t hq, hkv, group;
   int32_t stream_keys;                 // tensor-core kernel: keys are the first to leave L2
   int32_t causal;                      // APACK_SOFTMAX_CAUSAL_ROW: row r of n_q sees keys <= q_pos + r

@@ -501,8 +501,6 @@ apack_status run_score_narrow(const apack_seqs *seqs, const void *q, const void 
       max_nparts = std::max(max_nparts, sq.nparts);
       max_parts = std::max(max_parts, static_cast<int64_t>(sq.rows) * sq.nparts);
     }
-    P.total_units = units;
-    P.total_units8 = units8;
     if (units == 0) continue;
     const uint16_t *q16 = static_cast<const uint16_t *>(q);
     const uint8_t *k8 = static_cast<const uint8_t *>(k);
