@@ -460,13 +460,17 @@ int64_t decode_chunks(int32_t num_seqs, const int32_t *cu_seqlens_h, int chunk) 
 }
 
 // Chunks of this batch or of one with shorter caches, at most: decode_chunk_keys leaves a launch one CTA per
-// SM, or one chunk per sequence (of kMaxChunkKeys keys).  Fewer keys can mean more chunks (152 SMs: 19,456
-// keys 152 chunks, 19,457 keys 77), so a workspace for the longest caches needs the bound, not their count.
+// SM, or one chunk per sequence (of kMaxChunkKeys keys), and a chunk has 128 keys or is its sequence's last.
+// Fewer keys can mean more chunks (152 SMs: 19,456 keys 152 chunks, 19,457 keys 77), so a workspace for the
+// longest caches needs the bound, not their count.
 int64_t decode_chunks_bound(int32_t num_seqs, const int32_t *cu_seqlens_h) {
   int64_t bound = 0;
-  for (int s0 = 0; s0 < num_seqs; s0 += kSeqsPerLaunch)
-    bound += std::max<int64_t>(device_sm_count(), decode_chunks(std::min(num_seqs - s0, kSeqsPerLaunch),
-                                                                cu_seqlens_h + s0, static_cast<int>(kMaxChunkKeys)));
+  for (int s0 = 0; s0 < num_seqs; s0 += kSeqsPerLaunch) {
+    const int ns = std::min(num_seqs - s0, kSeqsPerLaunch);
+    const int64_t one_round = std::max<int64_t>(
+        device_sm_count(), decode_chunks(ns, cu_seqlens_h + s0, static_cast<int>(kMaxChunkKeys)));
+    bound += std::min(one_round, decode_chunks(ns, cu_seqlens_h + s0, 128));
+  }
   return bound;
 }
 
